@@ -77,7 +77,7 @@ int choose_fft_size(int n) {
     return best;
 }
 
-// Twiddle arrays of 3 L entries: [0, L) the natural table exp(-2 pi i m / L); for
+// Twiddle arrays (FP64: the natural table only; complex64: 3 L entries): [0, L) the natural table exp(-2 pi i m / L); for
 // L = 2^a in [256, 4096] (the compile-time stages of fft_fast.cuh), [L, 2 L) and
 // [2 L, 3 L) the stage tables of the forward and inverse plans: stage s (radix R,
 // sub-transform length Ns) keeps at r Ns + k - 1 (1 <= r < R, k < Ns) the natural entry
@@ -95,22 +95,28 @@ static void stage_table(int L, bool inv, const V* nat, V* out) {
     }
 }
 
-static void twiddles(int L, std::vector<double2>& d, std::vector<float2>& f) {
-    d.assign(3 * (size_t)L, make_double2(0.0, 0.0));
+static void twiddles(int L, std::vector<double2>& d, std::vector<float2>& f, std::vector<fxw>& w) {
+    d.assign((size_t)L, make_double2(0.0, 0.0));
+    std::vector<fxw> nat(L);
     f.assign(3 * (size_t)L, make_float2(0.f, 0.f));
     const long double two_pi = 6.283185307179586476925286766559005768L;
     for (int m = 0; m < L; m++) {
         const long double ang = two_pi * (long double)m / (long double)L;
-        const double c = (double)cosl(ang), s = -(double)sinl(ang);
+        const long double cl = cosl(ang), sl = -sinl(ang);
+        const double c = (double)cl, s = (double)sl;
+        nat[m] = fx_factor(cl, sl);
         d[m] = make_double2(c, s);
         f[m] = make_float2((float)c, (float)s);
     }
     if (L >= 256 && L <= 4096 && (L & (L - 1)) == 0) {
-        for (int inv = 0; inv < 2; inv++) {
-            stage_table(L, inv != 0, d.data(), d.data() + (1 + inv) * (size_t)L);
-            stage_table(L, inv != 0, f.data(), f.data() + (1 + inv) * (size_t)L);
-        }
+        for (int inv = 0; inv < 2; inv++) stage_table(L, inv != 0, f.data(), f.data() + (1 + inv) * (size_t)L);
     }
+    // factors of the fixed-point plan (fx.cuh): stage (R, Ns) at r Ns + k - 1
+    w.assign((size_t)L, fxw{0, 0, 0, 0});
+    const FxPlan p = fx_plan(L);
+    for (int s = 1, ns = p.r0; s <= p.q; ns *= p.r1, s++)
+        for (int r = 1; r < p.r1; r++)
+            for (int k = 0; k < ns; k++) w[r * ns + k - 1] = nat[(long)(L / (ns * p.r1)) * r * k];
 }
 
 static std::atomic<uint64_t> g_next_id{1};
@@ -122,7 +128,8 @@ using namespace die;
 
 static void free_op(dieop_s* op) {
     if (!op) return;
-    void* ptrs[] = {op->tw1_d, op->tw2_d, op->tw1_f, op->tw2_f, op->gq_d, op->gq_f, op->chi_d, op->chir_d,
+    void* ptrs[] = {op->tw1_d, op->tw2_d, op->tw1_f, op->tw2_f, op->fx1, op->fx2, op->gx, op->ge, op->gq_f,
+                    op->chi_d, op->chir_d,
                     op->chi_f, op->chir_f, op->chim_d, op->chim_f, op->ws.W, op->ws.v, op->wsb.W, op->wsb.v,
                     op->dflag};
     for (void* p : ptrs)
@@ -290,12 +297,15 @@ static die_status create_impl(const dieop_desc* desc, const void* eps_r, int eps
     op->Q2 = op->M2 / 2 + 1;
     DIE_CUDA_TRY(cudaGetDevice(&op->device));
     const long N = op->N, q = (long)op->Q1 * op->Q2;
-    DIE_TRY(dmalloc(&op->tw1_d, 3 * (size_t)op->M1 * sizeof(double2)));
-    DIE_TRY(dmalloc(&op->tw2_d, 3 * (size_t)op->M2 * sizeof(double2)));
+    DIE_TRY(dmalloc(&op->tw1_d, (size_t)op->M1 * sizeof(double2)));
+    DIE_TRY(dmalloc(&op->tw2_d, (size_t)op->M2 * sizeof(double2)));
+    DIE_TRY(dmalloc(&op->fx1, (size_t)op->M1 * sizeof(fxw)));
+    DIE_TRY(dmalloc(&op->fx2, (size_t)op->M2 * sizeof(fxw)));
     DIE_TRY(dmalloc(&op->tw1_f, 3 * (size_t)op->M1 * sizeof(float2)));
     DIE_TRY(dmalloc(&op->tw2_f, 3 * (size_t)op->M2 * sizeof(float2)));
     const int ng = green_plane_count(op);
-    DIE_TRY(dmalloc(&op->gq_d, ng * q * sizeof(double2)));
+    DIE_TRY(dmalloc(&op->gx, ng * q * sizeof(fxw)));
+    DIE_TRY(dmalloc(&op->ge, op->Q1 * sizeof(int)));
     DIE_TRY(dmalloc(&op->gq_f, ng * q * sizeof(float2)));
     DIE_TRY(dmalloc(&op->chi_d, N * sizeof(double2)));
     DIE_TRY(dmalloc(&op->chir_d, N * sizeof(double2)));
@@ -317,8 +327,11 @@ static die_status create_impl(const dieop_desc* desc, const void* eps_r, int eps
 
     std::vector<double2> t1d, t2d;
     std::vector<float2> t1f, t2f;
-    twiddles(op->M1, t1d, t1f);
-    twiddles(op->M2, t2d, t2f);
+    std::vector<fxw> x1, x2;
+    twiddles(op->M1, t1d, t1f, x1);
+    twiddles(op->M2, t2d, t2f, x2);
+    DIE_CUDA_TRY(cudaMemcpyAsync(op->fx1, x1.data(), x1.size() * sizeof(fxw), cudaMemcpyHostToDevice, st));
+    DIE_CUDA_TRY(cudaMemcpyAsync(op->fx2, x2.data(), x2.size() * sizeof(fxw), cudaMemcpyHostToDevice, st));
     DIE_CUDA_TRY(cudaMemcpyAsync(op->tw1_d, t1d.data(), t1d.size() * sizeof(double2), cudaMemcpyHostToDevice, st));
     DIE_CUDA_TRY(cudaMemcpyAsync(op->tw2_d, t2d.data(), t2d.size() * sizeof(double2), cudaMemcpyHostToDevice, st));
     DIE_CUDA_TRY(cudaMemcpyAsync(op->tw1_f, t1f.data(), t1f.size() * sizeof(float2), cudaMemcpyHostToDevice, st));

@@ -1,0 +1,8 @@
+// FP64 product passes (fx_kernels.cuh): length 2048.
+#include "fx_kernels.cuh"
+
+namespace die {
+
+template struct FxLaunch<16, fx_plan(2048).r0, fx_plan(2048).r1, 2048>;
+
+}  // namespace die

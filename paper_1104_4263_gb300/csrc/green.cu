@@ -143,6 +143,34 @@ __global__ void quarter_kernel(const double2* __restrict__ spec, int nplanes, in
     }
 }
 
+// Quarter spectra to fixed point, in place (one block per k1q): one scale for the planes of
+// a k1q, such that the sum over a column's planes of the magnitudes stays within 2^63.
+__global__ void green_fixed_kernel(double2* gq, int nplanes, int Q1, int Q2, int* ge) {
+    __shared__ int s_e;
+    if (threadIdx.x == 0) s_e = 0;
+    __syncthreads();
+    const long plane = (long)Q1 * Q2;
+    double2* g = gq + (long)blockIdx.x * Q2;
+    int e = 0;
+    for (int i = threadIdx.x; i < nplanes * Q2; i += blockDim.x) {
+        const double2 v = g[(i / Q2) * plane + i % Q2];
+        e = max(e, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff) >> 20);
+    }
+    atomicMax(&s_e, e);
+    __syncthreads();
+    const int f = (nplanes > 3 ? 60 : 61) - (s_e - 1022);     // |component| < 2^(s_e - 1022)
+    for (int i = threadIdx.x; i < nplanes * Q2; i += blockDim.x) {
+        double2* p = &g[(i / Q2) * plane + i % Q2];
+        const double2 v = *p;
+        fxw w;
+        fx_split(__double2ll_rn(scalbn(v.x, f)), w.xh, w.xl);
+        fx_split(__double2ll_rn(scalbn(v.y, f)), w.yh, w.yl);
+        if (w.yl == INT_MIN) w.yl++;
+        *reinterpret_cast<fxw*>(p) = w;
+    }
+    if (threadIdx.x == 0) ge[blockIdx.x] = f - 63;
+}
+
 static die_status fft_lines(double2* data, long elem_stride, long line_stride, int nlines, const FftPlan& pl,
                             const double2* tw, cudaStream_t st) {
     const int G = pl.L / pl.ept;
@@ -170,8 +198,10 @@ die_status build_green_spectrum(dieop_s* op, double2* scratch, cudaStream_t st) 
         DIE_TRY(fft_lines(base, 1, M1, M2, op->f1, op->tw1_d, st));       // rows: along x1
         DIE_TRY(fft_lines(base, M1, 1, M1, op->f2, op->tw2_d, st));       // columns: along x2
     }
-    quarter_kernel<<<1216, 256, 0, st>>>(scratch, nplanes, M1, M2, op->Q1, op->Q2, 1.0 / ((double)M1 * M2), op->gq_d,
-                                         op->gq_f);
+    quarter_kernel<<<1216, 256, 0, st>>>(scratch, nplanes, M1, M2, op->Q1, op->Q2, 1.0 / ((double)M1 * M2),
+                                         reinterpret_cast<double2*>(op->gx), op->gq_f);
+    DIE_LAUNCH_CHECK();
+    green_fixed_kernel<<<op->Q1, 256, 0, st>>>(reinterpret_cast<double2*>(op->gx), nplanes, op->Q1, op->Q2, op->ge);
     DIE_LAUNCH_CHECK();
     return DIE_OK;
 }

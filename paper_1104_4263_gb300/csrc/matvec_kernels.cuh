@@ -1,6 +1,6 @@
 // FFT-speed products with the discretised TE operator A = I - G X (Eqs. (4.3)-(4.5)):
-// kernels and launchers, included by the instantiation units matvec.cu (FP64) and
-// matvec_f32.cu (complex64 arithmetic).
+// kernels and launchers of the complex64 products, instantiated in matvec_f32.cu (the FP64
+// products run the same passes in fixed point, fx_kernels.cuh).
 //
 // G is block-Toeplitz (its entries depend on x_n - x_m only), so G w is a 2-D
 // linear convolution of the 2 x 2 Green's tensor table with the contrast current
@@ -35,7 +35,7 @@
 namespace die {
 
 // Rows per block of the row passes: enough for 32-byte segments in the transposed
-// accesses (4 complex64 / 2 complex128), at most 512 threads per block.
+// accesses (4 complex64), at most 512 threads per block.
 template <typename C> constexpr int tile_rows() { return sizeof(C) == 8 ? 4 : 2; }
 constexpr size_t kStageGreenMaxSmem = 200 * 1024;
 
@@ -425,14 +425,10 @@ template <int L> constexpr int tile_stride_c() { return L + (L >> 4) + 2; }
 template <typename C>
 __device__ __forceinline__ void cp_async_elem(C* smem, const C* gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    if constexpr (sizeof(C) == 8) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
-    else asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
+    static_assert(sizeof(C) == 8, "complex64");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-// Blocks per SM that the column pass should fit: all M1 = 1024 complex64 columns in one
-// wave of 152 SMs needs 7 (at most 72 registers per thread).
-template <typename C, int L> constexpr int k2_min_blocks() { return (sizeof(C) == 8 && L == 1024) ? 7 : 1; }
 
 // Transposed tile I/O of the row passes: thread (k0 = tid / TR, r = tid % TR) moves
 // elements k1 = k0 + it G, it < 16, of tile row r.
@@ -576,91 +572,6 @@ __global__ void __launch_bounds__(512) k1_defl_fast(OpDev<float> op, DeflIn d, c
     __syncthreads();
     run_fast<C, L, false, 1, P2<L>::fwd.ns, false>(buf, x, t, op.twx1, active);
     tile_io<C, L, TR, true>(tile, W, c, i2_0, op.n2);
-}
-
-template <typename T, int L>
-__global__ void __launch_bounds__(2 * (L / 16), k2_min_blocks<C_t<T>, L>()) k2_fast(OpDev<T> op, C_t<T>* __restrict__ W,
-                                                                                 int stage_g, const int* __restrict__ skip) {
-    using C = C_t<T>;
-    constexpr int G = L / 16, n2 = L / 2, Q2 = L / 2 + 1, Lp = L + (L >> 4);
-    constexpr int nsf = P2<L>::fwd.ns, nsi = P2<L>::inv.ns;
-    using F0 = typename PlanStage<C, L, false, 0>::St;
-    using I0 = typename PlanStage<C, L, true, 0>::St;
-    using IL = typename PlanStage<C, L, true, nsi - 1>::St;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* buf0 = reinterpret_cast<C*>(smem_raw);
-    C* buf1 = buf0 + Lp;
-    C* gs = buf1 + Lp;
-    const int comp = threadIdx.x >= G ? 1 : 0;
-    const int t = threadIdx.x - comp * G;
-    C* buf = comp ? buf1 : buf0;
-    W += blockIdx.y * op.ws;            // right-hand side of a batched product
-    const int k1 = blockIdx.x;
-    C* col = W + ((long)comp * op.M1 + k1) * n2 + t;
-    const int h1 = op.M1 >> 1;
-    const int k1q = k1 <= h1 ? k1 : op.M1 - k1;
-    const bool neg1 = k1 > h1;
-    const long plane = (long)op.Q1 * Q2;
-    const C* g = op.gq + (long)k1q * Q2;
-    if (stage_g) {   // the column's three quarter-spectrum rows (operator constants), issued
-                     // before the wait on the previous kernel; they land during the forward FFT
-        for (int e = threadIdx.x; e < 3 * Q2; e += 2 * G) {
-            const int pl = e / Q2, q = e - pl * Q2;
-            cp_async_elem(gs + e, g + pl * plane + q);
-        }
-    }
-    pdl_wait();
-    if (block_flag(skip)) {
-        cp_async_wait_all();
-        return;
-    }
-    C x[16];
-#pragma unroll
-    for (int e = 0; e < 16; e++) {
-        const int idx = F0::index(e);
-        x[e] = idx < n2 ? col[idx] : czero<C>();
-    }
-    F0::compute(x, t, op.twx2);
-    F0::store(buf, x, t);
-    __syncthreads();
-    run_fast<C, L, false, 1, nsf, false>(buf, x, t, op.twx2, true);
-    if (stage_g) {
-        cp_async_wait_all();
-        __syncthreads();
-    }
-    {   // 2 x 2 Green-spectrum multiply at the first inverse stage's indices k2 = t + c
-        const long ps = stage_g ? (long)Q2 : plane;
-        const C* gsrc = stage_g ? gs : g;
-        const C* gdp = gsrc + comp * ps + t;     // k2 <= L/2: quarter index k2
-        const C* gop = gsrc + 2 * ps + t;
-        const C* gdm = gsrc + comp * ps - t;     // k2 > L/2: quarter index L - k2
-        const C* gom = gsrc + 2 * ps - t;
-        const C* a0 = buf0 + pidx(t);
-        const C* a1 = buf1 + pidx(t);
-#pragma unroll
-        for (int e = 0; e < 16; e++) {
-            const int c = I0::index(e);
-            const C a = a0[c + (c >> 4)], b = a1[c + (c >> 4)];
-            C gd, go;
-            bool neg2;
-            if (c < L / 2) { gd = gdp[c]; go = gop[c]; neg2 = false; }
-            else { gd = gdm[L - c]; go = gom[L - c]; neg2 = c > L / 2 || t > 0; }
-            if (neg1 != neg2) { go.x = -go.x; go.y = -go.y; }
-            x[e] = comp == 0 ? cadd(cmul(gd, a), cmul(go, b)) : cadd(cmul(go, a), cmul(gd, b));
-        }
-    }
-    __syncthreads();
-    I0::compute(x, t, op.twx2);
-    I0::store(buf, x, t);
-    __syncthreads();
-    run_fast<C, L, true, 1, nsi - 1, false>(buf, x, t, op.twx2, true);
-    IL::load(buf, x, t);
-    IL::compute(x, t, op.twx2);
-#pragma unroll
-    for (int e = 0; e < 16; e++) {
-        const int idx = IL::index(e);
-        if (idx < n2) col[idx] = x[e];
-    }
 }
 
 // Complex64 column pass with both components in the same thread (G threads per column):
@@ -1000,16 +911,10 @@ inline void launch_k2(const OpDev<T>& v, C_t<T>* W, const int* skip, cudaStream_
         return;
     }
     if (fast_cols(v)) {
-        if constexpr (sizeof(C_t<T>) == 8) {     // complex64: both components per thread
-            const Launch l2{l.grid, dim3(v.M2 / 16), l.smem};
+        const Launch l2{l.grid, dim3(v.M2 / 16), l.smem};     // both components per thread
 #define K2F_CASE(LSV) { static std::atomic<bool> a_{false}; launch_kernel(k2_fast2<T, LSV>, a_, l2, st, v, W, sg, skip); }
-            DIE_PROF(PK_COLS, st, DIE_FAST_SWITCH(v.M2, K2F_CASE));
+        DIE_PROF(PK_COLS, st, DIE_FAST_SWITCH(v.M2, K2F_CASE));
 #undef K2F_CASE
-        } else {
-#define K2F_CASE(LSV) { static std::atomic<bool> a_{false}; launch_kernel(k2_fast<T, LSV>, a_, l, st, v, W, sg, skip); }
-            DIE_PROF(PK_COLS, st, DIE_FAST_SWITCH(v.M2, K2F_CASE));
-#undef K2F_CASE
-        }
         return;
     }
 #define K2_CASE(LSV) { static std::atomic<bool> a_{false}; launch_kernel(k2_cols<T, 16, LSV>, a_, l, st, v, W, sg, skip); }
@@ -1058,10 +963,6 @@ inline void launch_k3k1(const OpDev<T>& v, C_t<T>* W, const IO* u, const C_t<T>*
 }
 
 template <typename T> struct Sel;
-template <> struct Sel<double> {
-    static const double2* chi(const dieop_s* o, Contrast c) { return c == Contrast::Chi ? o->chi_d : o->chir_d; }
-    static OpDev<double> view(const dieop_s* o) { return view_d(o); }
-};
 template <> struct Sel<float> {
     static const float2* chi(const dieop_s* o, Contrast c) { return c == Contrast::Chi ? o->chi_f : o->chir_f; }
     static OpDev<float> view(const dieop_s* o) { return view_f(o); }

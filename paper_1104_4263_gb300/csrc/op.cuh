@@ -2,7 +2,7 @@
 #pragma once
 
 #include "common.cuh"
-#include "fft.cuh"
+#include "fx.cuh"
 
 namespace die {
 
@@ -55,10 +55,13 @@ struct dieop_s {
     die_precision prec = DIE_FP64;
     die_polarization pol = DIE_TE;
     die::FftPlan f1{}, i1{}, f2{}, i2{};
-    double2 *tw1_d = nullptr, *tw2_d = nullptr;   // 3 M entries: natural table, then the
-    float2 *tw1_f = nullptr, *tw2_f = nullptr;    // forward and inverse stage tables
+    double2 *tw1_d = nullptr, *tw2_d = nullptr;   // M entries: natural table (set-up only)
+    float2 *tw1_f = nullptr, *tw2_f = nullptr;    // 3 M entries: natural table, then the
+                                                  // forward and inverse stage tables
+    die::fxw *fx1 = nullptr, *fx2 = nullptr;      // M entries: factors of the fixed-point plans
     int planes = 2;                // field planes: 3 for DIE_TE_MAG (E1, E2, H3)
-    double2* gq_d = nullptr;       // (planes == 3 ? 6 : 3) * Q1 * Q2
+    die::fxw* gx = nullptr;        // (planes == 3 ? 6 : 3) * Q1 * Q2, fixed point, one scale
+    int* ge = nullptr;             // (exponent ge + 63) per k1q: Q1 entries
     float2* gq_f = nullptr;
     double2 *chi_d = nullptr, *chir_d = nullptr;   // chi = eps_r - 1, chi' = 1/eps_r - 1
     float2 *chi_f = nullptr, *chir_f = nullptr;
@@ -82,7 +85,6 @@ inline int green_plane_count(const dieop_s* op) { return op->planes == 3 ? 6 : 3
 // Complex entries of one field vector.
 inline long vec_len(const dieop_s* op) { return (long)op->planes * op->N; }
 
-OpDev<double> view_d(const dieop_s* op);
 OpDev<float> view_f(const dieop_s* op);
 
 enum class Contrast { Chi, ChiReg };

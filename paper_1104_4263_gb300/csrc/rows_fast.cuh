@@ -1,6 +1,6 @@
 // Launchers of the fast row passes at one tile height TR (declared in matvec_kernels.cuh).
 // A translation unit that includes this header instantiates the launchers of one height
-// (DIE_INSTANTIATE_ROWS_C64 / _C128), so that the kernels of each height are compiled
+// (DIE_INSTANTIATE_ROWS_C64), so that the kernels of each height are compiled
 // once, in parallel with the others.
 #pragma once
 
@@ -88,17 +88,4 @@ void rows_defl_fast(const OpDev<float>& v, const DeflIn& d, const float2* chi, f
                                                         const float2*, float2*, const int*, cudaStream_t, int); \
     template void rows_defl_fast<TR>(const OpDev<float>&, const DeflIn&, const float2*, float2*, float2*,     \
                                      const int*, cudaStream_t);                                              \
-    }
-
-// The FP64 products (default height only).
-#define DIE_INSTANTIATE_ROWS_C128                                                                             \
-    namespace die {                                                                                          \
-    template void rows_fwd_fast<double, double2, 0>(const OpDev<double>&, const double2*, const double2*,    \
-                                                    double2*, const int*, cudaStream_t, int);               \
-    template void rows_inv_fast<double, double2, double2, 0>(const OpDev<double>&, const double2*,           \
-                                                             const double2*, double2*, const int*,          \
-                                                             cudaStream_t, int);                            \
-    template void rows_inv_fwd_fast<double, double2, 0>(const OpDev<double>&, double2*, const double2*,      \
-                                                        const double2*, double2*, const int*, cudaStream_t,  \
-                                                        int);                                                \
     }
