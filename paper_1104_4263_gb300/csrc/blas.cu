@@ -78,19 +78,24 @@ __device__ __forceinline__ void block_partials(A (&acc)[K], A* red, int g0, cons
     __syncthreads();
 }
 
-// Final sums of the per-block partials partial[i * gridDim.x + b], i < nv (see
-// RedScratch).  Every thread of every block calls it after its block's partials are
-// written; it returns true in the one block that has written out[0 .. nv), whose
-// threads may then read out.
-__device__ bool reduce_partials(const RedScratch& rs, int nv, double2* out) {
+// Final sums of the per-block partials partial[i * gridDim.x + b] (see RedScratch) of the
+// vectors this block's row of the grid works on: all i < nv, or, when gridDim.y > 1, the
+// groups y, y + gridDim.y, ... of gv vectors.  Every thread of every block calls it after its
+// block's partials are written; it returns true in the one block (of each grid row) that
+// has written their sums to out, whose threads may then read them.
+__device__ bool reduce_partials(const RedScratch& rs, int nv, double2* out, int gv = kMaxBasis) {
     __shared__ int s_last;
     const int G = gridDim.x, ng = (G + kRedGroup - 1) / kRedGroup, g = blockIdx.x / kRedGroup;
     const int gsz = min(kRedGroup, G - g * kRedGroup);
+    const int y = blockIdx.y, gy = gridDim.y;
+    unsigned* counter = rs.counter + y * (1 + kRedGroupsMax);
+    const int nl = gy == 1 ? nv : ((nv + gv - 1) / gv - y + gy - 1) / gy * gv;   // local vector slots
+    auto vec = [&](int l) { return gy == 1 ? l : (l / gv * gy + y) * gv + l % gv; };
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
-        const bool last = atomicAdd(&rs.counter[1 + g], 1u) == (unsigned)(gsz - 1);
-        if (last) rs.counter[1 + g] = 0;
+        const bool last = atomicAdd(&counter[1 + g], 1u) == (unsigned)(gsz - 1);
+        if (last) counter[1 + g] = 0;
         s_last = last;
     }
     __syncthreads();
@@ -98,28 +103,32 @@ __device__ bool reduce_partials(const RedScratch& rs, int nv, double2* out) {
     __threadfence();
     const double* pp = reinterpret_cast<const double*>(rs.partial);
     double* p2 = reinterpret_cast<double*>(rs.partial2);
-    for (int e = threadIdx.x; e < 2 * nv; e += blockDim.x) {   // e = 2 i + component
-        const double* src = pp + 2 * ((long)(e >> 1) * G + (long)g * kRedGroup) + (e & 1);
+    for (int e = threadIdx.x; e < 2 * nl; e += blockDim.x) {   // e = 2 l + component
+        const int i = vec(e >> 1);
+        if (i >= nv) continue;
+        const double* src = pp + 2 * ((long)i * G + (long)g * kRedGroup) + (e & 1);
         double s = 0;
         for (int b = 0; b < gsz; b++) s += __ldcg(src + 2 * b);
-        p2[2 * ((long)(e >> 1) * ng + g) + (e & 1)] = s;
+        p2[2 * ((long)i * ng + g) + (e & 1)] = s;
     }
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
-        const bool last = atomicAdd(&rs.counter[0], 1u) == (unsigned)(ng - 1);
-        if (last) rs.counter[0] = 0;
+        const bool last = atomicAdd(&counter[0], 1u) == (unsigned)(ng - 1);
+        if (last) counter[0] = 0;
         s_last = last;
     }
     __syncthreads();
     if (!s_last) return false;
     __threadfence();
     double* o = reinterpret_cast<double*>(out);
-    for (int e = threadIdx.x; e < 2 * nv; e += blockDim.x) {
-        const double* src = p2 + 2 * (long)(e >> 1) * ng + (e & 1);
+    for (int e = threadIdx.x; e < 2 * nl; e += blockDim.x) {
+        const int i = vec(e >> 1);
+        if (i >= nv) continue;
+        const double* src = p2 + 2 * (long)i * ng + (e & 1);
         double s = 0;
         for (int q = 0; q < ng; q++) s += __ldcg(src + 2 * q);
-        o[e] = s;
+        o[2 * i + (e & 1)] = s;
     }
     __syncthreads();
     return true;
@@ -266,12 +275,12 @@ __global__ void __launch_bounds__(kRedThreads, 2) proj3_kernel(const double2* __
     const bool off = block_flag(skip);
     if (off && !live) return;
     const int nvt = nv + (with_norm ? 1 : 0);
-    for (int g0 = 0; g0 < nvt; g0 += kGroup3) {
+    for (int g0 = blockIdx.y * kGroup3; g0 < nvt; g0 += gridDim.y * kGroup3) {
         if (off) { zero_partials(g0, 2 * kGroup3, nvt, rs); continue; }
         const int cnt = nvt - g0 < kGroup3 ? nvt - g0 : kGroup3;
         proj_group3_n<kGroup3>(cnt, V, VM, ldv, g0, nv, w, n, red, rs);
     }
-    reduce_partials(rs, nvt, out);
+    reduce_partials(rs, nvt, out, kGroup3);
 }
 
 // Runtime count -> compile-time CNT in [1, C].
@@ -296,12 +305,12 @@ __global__ void __launch_bounds__(kRedThreads) proj_kernel(const VT* __restrict_
     const bool off = block_flag(skip);
     if (off && !live) return;
     const int nvt = nv + (with_norm ? 1 : 0);
-    for (int g0 = 0; g0 < nvt; g0 += GV) {
+    for (int g0 = blockIdx.y * GV; g0 < nvt; g0 += gridDim.y * GV) {
         if (off) { zero_partials(g0, K, nvt, rs); continue; }
         const int cnt = nvt - g0 < GV ? nvt - g0 : GV;
         proj_group_n<VT, GV, false>(cnt, V, ldv, g0, nv, w, nullptr, nullptr, 1.0, n, red, rs);
     }
-    reduce_partials(rs, nvt, out);
+    reduce_partials(rs, nvt, out, GV);
 }
 
 // Deflation projections of the FP32-inner solves (see k_dots32): complex64 basis and
@@ -745,20 +754,50 @@ int red_blocks() {
     return b;
 }
 
-static inline int grid_for(long n) {
-    long b = (n + kRedThreads - 1) / kRedThreads;
+// Launch shape of a reduction over n rows: red_blocks() blocks of kRedThreads where that
+// leaves every thread a row; shorter vectors take smaller blocks, so that their rows still
+// spread over all SMs (the FP64 pipe of an SM does 2 operations per clock: 7442 rows in 29
+// blocks of 256 kept 123 SMs idle).  With red_rows: FP64 GMRES(40) at 61^2 288 -> 228 ms,
+// restart 400 at 133^2 313 -> 222 ms, eight solves at once at 64^2 167 -> 73 ms.
+struct RedShape { int blocks, threads; };
+static RedShape red_shape(long n) {
+    const int full = red_blocks();
+    const long per = (n + full - 1) / full;
+    if (per >= kRedThreads) return {full, kRedThreads};
+    const int threads = per <= 32 ? 32 : (int)((per + 31) / 32 * 32);
+    const long blocks = (n + threads - 1) / threads;
+    return {(int)(blocks < 1 ? 1 : blocks), threads};
+}
+// Rows of the grid that share the groups of gv among nvt vectors: one, unless short vectors
+// leave SMs with fewer than 32 warps; then groups run side by side instead of one after
+// another.
+static int red_rows(const RedShape& s, int nvt, int gv) {
+    const int groups = (nvt + gv - 1) / gv;
+    const long warps = (long)s.blocks * (s.threads / 32), room = 16l * red_blocks();   // 32 warps per SM
+    long y = room / warps;
+    if (y > groups) y = groups;
+    if (y > kRedRowsMax) y = kRedRowsMax;
+    return (int)(y < 1 ? 1 : y);
+}
+
+static inline int grid_for(long n, int threads = kRedThreads) {
+    long b = (n + threads - 1) / threads;
     return (int)(b < 1216 ? (b < 1 ? 1 : b) : 1216);
 }
+// Threads per block of the updates without a reduction (rows independent): as red_shape.
+static inline int axpy_threads(long n) { return red_shape(n).threads; }
 
 constexpr int kGroupFp64 = 8;        // FP64 projections per group (16 running sums per thread)
 
 die_status k_dots(const double2* V, long ldv, int nv, const double2* w, long n, int with_norm, double2* out,
                   const RedScratch& rs, const int* skip, cudaStream_t st, bool live, const double* VM) {
     if (nv + 1 > kMaxBasis || nv < 0) return DIE_EINVAL;
+    const RedShape sh = red_shape(n);
+    const int nvt = nv + (with_norm ? 1 : 0);
     if (VM)
-        DIE_PROF(PK_DOTS, st, launch_pdl(proj3_kernel, dim3(red_blocks()), dim3(kRedThreads), 0, st, V, VM, ldv, nv, w, n, with_norm, out, rs, skip, live ? 1 : 0));
+        DIE_PROF(PK_DOTS, st, launch_pdl(proj3_kernel, dim3(sh.blocks, red_rows(sh, nvt, kGroup3)), dim3(sh.threads), 0, st, V, VM, ldv, nv, w, n, with_norm, out, rs, skip, live ? 1 : 0));
     else
-        DIE_PROF(PK_DOTS, st, launch_pdl(proj_kernel<double2, kGroupFp64>, dim3(red_blocks()), dim3(kRedThreads), 0, st, V, ldv, nv, w, n, with_norm, out, rs, skip, live ? 1 : 0));
+        DIE_PROF(PK_DOTS, st, launch_pdl(proj_kernel<double2, kGroupFp64>, dim3(sh.blocks, red_rows(sh, nvt, kGroupFp64)), dim3(sh.threads), 0, st, V, ldv, nv, w, n, with_norm, out, rs, skip, live ? 1 : 0));
     DIE_LAUNCH_CHECK();
     return DIE_OK;
 }
@@ -777,10 +816,12 @@ die_status k_basis_axpy(const double2* V, long ldv, int k, const double2* coef, 
     const Dgks d = dec ? *dec : Dgks{};
     const int has_dec = dec && dec->reorth ? 1 : 0;
     if (nrm2) {
-        DIE_PROF(PK_UPDATE_NORM, st, launch_pdl(basis_axpy_kernel<double2, true>, dim3(red_blocks()), dim3(kRedThreads), 0, st,
+        const RedShape sh = red_shape(n);
+        DIE_PROF(PK_UPDATE_NORM, st, launch_pdl(basis_axpy_kernel<double2, true>, dim3(sh.blocks), dim3(sh.threads), 0, st,
                      V, ldv, k, coef, sign, (const double2*)nullptr, (const double2*)nullptr, base, out, n, nrm2, d, has_dec, rs, skip, live ? 1 : 0, VM));
     } else {
-        DIE_PROF(PK_LINCOMB, st, launch_pdl(basis_axpy_kernel<double2, false>, dim3(grid_for(n)), dim3(kRedThreads), 0, st,
+        const int t = axpy_threads(n);
+        DIE_PROF(PK_LINCOMB, st, launch_pdl(basis_axpy_kernel<double2, false>, dim3(grid_for(n, t)), dim3(t), 0, st,
                      V, ldv, k, coef, sign, (const double2*)nullptr, (const double2*)nullptr, base, out, n, (double2*)nullptr, d, 0, rs, skip, 0, VM));
     }
     DIE_LAUNCH_CHECK();
@@ -789,7 +830,8 @@ die_status k_basis_axpy(const double2* V, long ldv, int k, const double2* coef, 
 die_status k_defl_update(const double2* V, long ldv, int r, const double2* M, const double2* s, const double2* x,
                          double2* z, long n, const int* skip, cudaStream_t st) {
     if (r > kMaxBasis || r < 1) return DIE_EINVAL;
-    DIE_PROF(PK_DEFL_UPDATE, st, launch_pdl(basis_axpy_kernel<double2, false>, dim3(grid_for(n)), dim3(kRedThreads), 0, st,
+    const int t = axpy_threads(n);
+    DIE_PROF(PK_DEFL_UPDATE, st, launch_pdl(basis_axpy_kernel<double2, false>, dim3(grid_for(n, t)), dim3(t), 0, st,
                  V, ldv, r, (const double2*)nullptr, 1.0, M, s, x, z, n, (double2*)nullptr, Dgks{}, 0, RedScratch{}, skip, 0, (const double*)nullptr));
     DIE_LAUNCH_CHECK();
     return DIE_OK;
@@ -808,7 +850,8 @@ static die_status k_update_defl(const double2* V, long ldv, int k, const double2
                                 const int* skip, cudaStream_t st, bool live, const double* VM) {
     if (k > kMaxBasis || k < 0 || dp.r < 1 || dp.r > kDeflFoldMax) return DIE_EINVAL;
     const int ng = (dp.r + 7) / 8;
-#define UPD_CASE(NG) DIE_PROF(PK_UPDATE_NORM, st, launch_pdl(cgs_update_defl_kernel<NG>, dim3(red_blocks()), dim3(kRedThreads), 0, st, \
+    const RedShape sh = red_shape(n);
+#define UPD_CASE(NG) DIE_PROF(PK_UPDATE_NORM, st, launch_pdl(cgs_update_defl_kernel<NG>, dim3(sh.blocks), dim3(sh.threads), 0, st, \
                               V, ldv, k, coef, (const double2*)w, w, n, nrm2, dec, has_dec, dp, rs, skip, live ? 1 : 0, VM))
     switch (ng) {
         case 1: UPD_CASE(1); break;

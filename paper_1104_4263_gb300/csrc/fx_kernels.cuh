@@ -258,8 +258,8 @@ __device__ __forceinline__ void fx_store_tile(const double2* tile, double2* __re
 
 // ------------------------------------------------------------------------- K1
 template <int EPT, int R0, int R1, int LS>
-__global__ void __launch_bounds__(512) k1_fx(FxDev op, const double2* __restrict__ u, const double2* __restrict__ chi,
-                                             double2* __restrict__ W, const int* __restrict__ skip) {
+__global__ void __launch_bounds__(512) k1_fx(FxDev op, const double2* u, const double2* __restrict__ chi,
+                                             double2* __restrict__ W, FxNormalise nrm, const int* __restrict__ skip) {
     __shared__ FxNorm red[16];
     pdl_wait();
     if (block_flag(skip)) return;
@@ -273,10 +273,30 @@ __global__ void __launch_bounds__(512) k1_fx(FxDev op, const double2* __restrict
     const double2* urow = u + c * ((long)op.n1 * op.n2) + (long)i2 * op.n1;
     const double2* crow = (c == 2 ? op.chim : chi) + (long)i2 * op.n1;      // H3 plane: chi_m
     double2 z[EPT];
+    if (nrm.inv) {       // the basis vector's normalisation, in the pass that reads it anyway
+        const double sc = *nrm.inv;
+        const long off = urow - u;
 #pragma unroll
-    for (int e = 0; e < EPT; e++) {
-        const int j = fx_slot<EPT, R0>(e), idx = t + j * G;
-        z[e] = j < EPT / 2 && active && idx < op.n1 ? cmul(urow[idx], crow[idx]) : czero<double2>();
+        for (int e = 0; e < EPT; e++) {      // all loads before the first store
+            const int j = fx_slot<EPT, R0>(e), idx = t + j * G;
+            z[e] = j < EPT / 2 && active && idx < op.n1 ? urow[idx] : czero<double2>();
+        }
+#pragma unroll
+        for (int e = 0; e < EPT; e++) {
+            const int j = fx_slot<EPT, R0>(e), idx = t + j * G;
+            if (j < EPT / 2 && active && idx < op.n1) {
+                const double2 v = make_double2(z[e].x * sc, z[e].y * sc);
+                nrm.v[off + idx] = v;
+                if (nrm.vm) nrm.vm[off + idx] = v.x - v.y;
+                z[e] = cmul(v, crow[idx]);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < EPT; e++) {
+            const int j = fx_slot<EPT, R0>(e), idx = t + j * G;
+            z[e] = j < EPT / 2 && active && idx < op.n1 ? cmul(urow[idx], crow[idx]) : czero<double2>();
+        }
     }
     fx_row_forward<EPT, R0, R1, LS>(z, reinterpret_cast<fxc*>(smem_raw) + rs * Lp, op, t, G, L, red);
     __syncthreads();
@@ -483,10 +503,10 @@ static Launch fx_rows_launch(const FxDev& v, int ept, int nb) {
     return Launch{dim3((v.n2 + TR - 1) / TR, v.planes, nb), dim3(TR * G), (size_t)TR * tile_stride(v.M1) * sizeof(fxc)};
 }
 template <int EPT, int R0, int R1, int LS>
-void FxLaunch<EPT, R0, R1, LS>::k1(const FxDev& v, const double2* u, const double2* chi, double2* W, const int* skip,
-                                   cudaStream_t st, int nb) {
+void FxLaunch<EPT, R0, R1, LS>::k1(const FxDev& v, const double2* u, const double2* chi, double2* W,
+                                   const FxNormalise& nrm, const int* skip, cudaStream_t st, int nb) {
     static std::atomic<bool> a{false};
-    launch_kernel(k1_fx<EPT, R0, R1, LS>, a, fx_rows_launch(v, EPT, nb), st, v, u, chi, W, skip);
+    launch_kernel(k1_fx<EPT, R0, R1, LS>, a, fx_rows_launch(v, EPT, nb), st, v, u, chi, W, nrm, skip);
 }
 template <int EPT, int R0, int R1, int LS>
 void FxLaunch<EPT, R0, R1, LS>::k3(const FxDev& v, const double2* W, const double2* u, double2* y, const int* skip,

@@ -18,11 +18,19 @@ struct FxDev {
     int planes;
 };
 
+// First row pass of a product on a vector that is still to be normalised: v *= *inv in place
+// (v is the product's input), with Re - Im of the result in vm (or NULL).  inv NULL: as it is.
+struct FxNormalise {
+    double2* v = nullptr;
+    const double* inv = nullptr;
+    double* vm = nullptr;
+};
+
 // The passes at one transform length (LS) or, LS = 0, at the lengths R0 4^q; nb vectors per
 // launch.
 template <int EPT, int R0, int R1, int LS> struct FxLaunch {
-    static void k1(const FxDev& v, const double2* u, const double2* chi, double2* W, const int* skip,
-                   cudaStream_t st, int nb);
+    static void k1(const FxDev& v, const double2* u, const double2* chi, double2* W, const FxNormalise& nrm,
+                   const int* skip, cudaStream_t st, int nb);
     static void k2(const FxDev& v, double2* W, const int* skip, cudaStream_t st, int nb);
     static void k3(const FxDev& v, const double2* W, const double2* u, double2* y, const int* skip, cudaStream_t st,
                    int nb);

@@ -511,6 +511,9 @@ static die_status solve_ctx(dieop_s* op, defl_s* defl, const gmres_opts* o, cons
                 if (o->timing) DIE_CUDA_TRY(cudaEventRecord(c->ev[4 * j + 1], st));
                 DIE_TRY(reg ? apply_reg_skip_xy<float, float2, double2>(op, c->z32, w, S.done, st, pws)
                             : apply_op_skip_xy<float, float2, double2>(op, Contrast::Chi, c->z32, w, S.done, st, pws));
+            } else if (inv_prev && !defl && !mixed) {   // v_j normalised inside the first row pass
+                if (o->timing) DIE_CUDA_TRY(cudaEventRecord(c->ev[4 * j + 1], st));
+                DIE_TRY(apply_normalised(op, reg, vj, inv_prev, Vm ? Vm + (long)j * ldv : nullptr, w, S.done, st, pws));
             } else {
                 if (inv_prev) DIE_TRY(k_scale_by(vj, n, inv_prev, S.done, st, nullptr, Vm ? Vm + (long)j * ldv : nullptr));
                 const double2* src = vj;

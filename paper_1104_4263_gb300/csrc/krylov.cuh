@@ -15,9 +15,10 @@ constexpr int kRedThreads = 256;
 constexpr int kRedGroup = 16;        // blocks per first-level group of the final sums
 constexpr int kRedBlocksMax = 640;   // the reduction scratch holds partials of up to this many blocks
 constexpr int kRedGroupsMax = kRedBlocksMax / kRedGroup;
-// Blocks of every reduction launch: two per SM of the current device, a multiple of
-// kRedGroup (queried once per device).  The count is fixed for a device, so the
-// fixed-order sums are bitwise reproducible on it.
+constexpr int kRedRowsMax = 16;      // rows of a reduction's grid (groups of vectors side by side)
+// Most blocks of a reduction launch: two per SM of the current device, a multiple of
+// kRedGroup (queried once per device).  The launch shape depends on it, the vector length
+// and the number of vectors only, so the fixed-order sums are bitwise reproducible.
 int red_blocks();
 constexpr int kMaxBasis = 320;       // largest basis a single projection / update launch handles
 constexpr int kBasisChunk = 256;     // longer bases are swept in chunks of this many vectors
@@ -41,14 +42,14 @@ static_assert(kBasisChunk + 1 <= kMaxBasis, "a chunk and the norm fit the reduct
 // Reduction scratch.  Each block writes one partial per vector ([vector][block]); the
 // last block of each group of kRedGroup consecutive blocks to arrive sums the group's
 // partials in block order ([vector][group]); the last group to finish sums those in
-// group order.  The arrival counters (one per group, then the top one) are left at 0
-// by every kernel that uses them.
+// group order.  The arrival counters (one per group, then the top one, for each row of the
+// grid) are left at 0 by every kernel that uses them.
 struct RedScratch {
     double2* partial = nullptr;      // kMaxBasis * kRedBlocksMax
     double2* partial2 = nullptr;     // kMaxBasis * kRedGroupsMax
     unsigned* counter = nullptr;     // kRedCounters
 };
-constexpr int kRedCounters = 1 + kRedGroupsMax;
+constexpr int kRedCounters = kRedRowsMax * (1 + kRedGroupsMax);
 
 // DGKS decision taken by the last block of a norm-computing update: reorth = always ||
 // ||w'||^2 < eta^2 ||w||^2; skip2 = done || !reorth (makes the second pass return at once).

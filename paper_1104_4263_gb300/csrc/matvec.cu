@@ -57,13 +57,13 @@ static const double2* chi_of(const dieop_s* op, Contrast c) { return c == Contra
 
 // nb products (reg: A(chi') A(chi), else A(contrast)) over consecutive vectors.
 static die_status fx_product(dieop_s* op, bool reg, Contrast which, const double2* x, double2* y, double2* W,
-                             double2* vb, const int* skip, cudaStream_t st, int nb) {
+                             double2* vb, const int* skip, cudaStream_t st, int nb, const FxNormalise& nrm = {}) {
     const FxDev v = view_d(op);
     const double2* chi = chi_of(op, reg ? Contrast::Chi : which);
     auto cols = [&] {
         DIE_PROF(PK_COLS, st, fx_for_length(v.M2, [&](auto l) { l.k2(v, W, skip, st, nb); }));
     };
-    DIE_PROF(PK_ROWS_FWD, st, fx_for_length(v.M1, [&](auto l) { l.k1(v, x, chi, W, skip, st, nb); }));
+    DIE_PROF(PK_ROWS_FWD, st, fx_for_length(v.M1, [&](auto l) { l.k1(v, x, chi, W, nrm, skip, st, nb); }));
     cols();
     if (reg) {
         DIE_PROF(PK_ROWS_INV_FWD, st,
@@ -86,6 +86,11 @@ die_status apply_reg_skip<double, double2>(dieop_s* op, const double2* x, double
                                            cudaStream_t st, const Workspace* ws) {
     if (!ws) ws = &op->ws;
     return fx_product(op, true, Contrast::Chi, x, y, (double2*)ws->W, (double2*)ws->v, skip, st, 1);
+}
+die_status apply_normalised(dieop_s* op, bool reg, double2* x, const double* inv, double* xm, double2* y,
+                            const int* skip, cudaStream_t st, const Workspace* ws) {
+    if (!ws) ws = &op->ws;
+    return fx_product(op, reg, Contrast::Chi, x, y, (double2*)ws->W, (double2*)ws->v, skip, st, 1, {x, inv, xm});
 }
 template <>
 die_status apply_op<double, double2>(dieop_s* op, Contrast c, const double2* x, double2* y, cudaStream_t st,

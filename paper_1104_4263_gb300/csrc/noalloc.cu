@@ -18,7 +18,7 @@ constexpr long kNoAllocCounterSlots = (kRedCounters * sizeof(unsigned) + sizeof(
 // block partials | group partials | projections s | counters
 constexpr long kNoAllocSlots = kNoAllocPartials + kNoAllocPartials2 + kNoAllocMaxR + kNoAllocCounterSlots;
 
-// (128 * 640 + 128 * 40 + 128 + 11) * 16 bytes (about 1.4 MB), held by every GPU that
+// (128 * 640 + 128 * 40 + 128 + 164) * 16 bytes (about 1.4 MB), held by every GPU that
 // loads the library until the process exits.
 static __device__ __align__(256) double2 g_noalloc_scratch[kNoAllocSlots];
 

@@ -107,6 +107,11 @@ template <typename T, typename IO>
 die_status apply_reg_skip(dieop_s* op, const IO* x, IO* y, const int* skip, cudaStream_t st,
                           const Workspace* ws = nullptr);
 
+// FP64 product with Atilde (A_R A when reg, else A) of x normalised in the first row pass:
+// x *= *inv in place, xm (or NULL) = Re - Im of the result, y = Atilde x.  y != x.
+die_status apply_normalised(dieop_s* op, bool reg, double2* x, const double* inv, double* xm, double2* y,
+                            const int* skip, cudaStream_t st, const Workspace* ws = nullptr);
+
 // nb products over consecutive field vectors, with a workspace of nb sets of row spectra
 // (Wws) and nb middle vectors (vws, used when reg).
 template <typename T, typename IO>
