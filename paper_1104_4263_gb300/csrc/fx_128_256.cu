@@ -3,7 +3,7 @@
 
 namespace die {
 
-template struct FxLaunch<16, fx_plan(128).r0, fx_plan(128).r1, 128>;
-template struct FxLaunch<16, fx_plan(256).r0, fx_plan(256).r1, 256>;
+template struct FxLaunch<fx_plan(128).ept, fx_plan(128).r0, fx_plan(128).r1, 128>;
+template struct FxLaunch<fx_plan(256).ept, fx_plan(256).r0, fx_plan(256).r1, 256>;
 
 }  // namespace die

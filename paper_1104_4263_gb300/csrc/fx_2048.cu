@@ -3,6 +3,6 @@
 
 namespace die {
 
-template struct FxLaunch<16, fx_plan(2048).r0, fx_plan(2048).r1, 2048>;
+template struct FxLaunch<fx_plan(2048).ept, fx_plan(2048).r0, fx_plan(2048).r1, 2048>;
 
 }  // namespace die

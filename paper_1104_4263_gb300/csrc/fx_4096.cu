@@ -3,6 +3,6 @@
 
 namespace die {
 
-template struct FxLaunch<16, fx_plan(4096).r0, fx_plan(4096).r1, 4096>;
+template struct FxLaunch<fx_plan(4096).ept, fx_plan(4096).r0, fx_plan(4096).r1, 4096>;
 
 }  // namespace die

@@ -3,7 +3,7 @@
 
 namespace die {
 
-template struct FxLaunch<16, fx_plan(512).r0, fx_plan(512).r1, 512>;
-template struct FxLaunch<16, fx_plan(1024).r0, fx_plan(1024).r1, 1024>;
+template struct FxLaunch<fx_plan(512).ept, fx_plan(512).r0, fx_plan(512).r1, 512>;
+template struct FxLaunch<fx_plan(1024).ept, fx_plan(1024).r0, fx_plan(1024).r1, 1024>;
 
 }  // namespace die

@@ -5,8 +5,9 @@
 // What bounds them: instruction issue and, on one wave of blocks, the serial chain of a
 // thread (the FP64 forms were bound by the FP64 pipe).  CUDA-event times per launch, FP64
 // form -> this one: 512^2 K1 82.5 -> 29.6 us, K2 290.6 -> 66.2, K3K1 155.5 -> 45.0, K3
-// 79.8 -> 26.5 (the regularised product 878 -> 210 us back to back); 61^2 128 -> 70 us; the
-// three-plane product at 384^2 476 -> 132 us.  A product's own rounding (spread of
+// 79.8 -> 26.5 (the regularised product 878 -> 207 us back to back); 61^2 128 -> 44 us; the
+// three-plane product at 384^2 476 -> 132 us.  Lengths 3 * 2^a have compile-time plans from
+// 48 to 1536 (runtime -> compile time: 96^2 83 -> 61 us, 700^2 700 -> 563).  A product's own rounding (spread of
 // y(c x) / c over random factors c) is 3.2e-16 ... 3.9e-16 of it at 61^2 ... 2048 x 1500 on
 // noise and wave fields, against 3.5e-16 ... 3.8e-16 of the FP64 form, and 3.3e-16 ...
 // 3.9e-16 against 3.9e-16 ... 4.4e-16 for regularised products.
@@ -180,8 +181,7 @@ __device__ __forceinline__ void fx_transform(fxc (&x)[EPT], fxc* buf, int q, con
         int Ns = R0, room = 0;
         const bool rise = q > 1 && !sc.bad;
         if (rise) room = fx_room(R0, R1, q, sc.half, sc.lm, sc.ls, 0);
-#pragma unroll 1
-        for (int s = 1;; s++) {
+        auto stage = [&](int s) {
             stage_load<fxc, EPT, R1>(buf, x, L, t, G);
             if (rise && s > 1) {
                 const int to = fx_room(R0, R1, q, sc.half, sc.lm, sc.ls, s - 1);
@@ -195,10 +195,17 @@ __device__ __forceinline__ void fx_transform(fxc (&x)[EPT], fxc* buf, int q, con
             }
             fx_stage<EPT, R1>(x, Ns, t, G, tw);
             __syncthreads();
-            if (s == q) break;
+            if (s == q) return;
             stage_store<fxc, EPT, R1>(buf, x, L, Ns, t, G);
             __syncthreads();
             Ns *= R1;
+        };
+        if constexpr (LS != 0 && R1 == 4) {       // short stages, Ns = 3 * 2^b: divisions by constants
+#pragma unroll
+            for (int s = 1; s <= fx_plan(LS ? LS : 16).q; s++) stage(s);
+        } else {
+#pragma unroll 1
+            for (int s = 1; s <= q; s++) stage(s);
         }
         sc.e -= 2 * q;
     }
@@ -393,11 +400,13 @@ __global__ void __launch_bounds__(512) k3k1_fx(FxDev op, double2* __restrict__ W
 // One block per column k1, G threads per plane.  One scale for the planes of the column
 // (their products are added), raised to the largest value before the Green multiply and
 // chosen anew for each plane's inverse transform.
-// Blocks per SM that keep a thread's registers at 128: 16 warps.
-constexpr int fx_k2_blocks(int threads) { return threads <= 512 ? 16 / ((threads + 31) / 32) : 1; }
+// Blocks per SM that keep a thread's registers at 128 (16 warps), or at 80 with 8 values.
+constexpr int fx_k2_blocks(int threads, int ept) {
+    return threads <= 512 ? (ept == 8 ? 24 : 16) / ((threads + 31) / 32) : 1;
+}
 
 template <int P, int EPT, int R0, int R1, int LS, int MAXT>
-__global__ void __launch_bounds__(MAXT, fx_k2_blocks(MAXT)) k2_fx(FxDev op, double2* __restrict__ W, const int* __restrict__ skip) {
+__global__ void __launch_bounds__(MAXT, fx_k2_blocks(MAXT, EPT)) k2_fx(FxDev op, double2* __restrict__ W, const int* __restrict__ skip) {
     constexpr int RL = fx_last<R0, R1, LS>();
     __shared__ FxNorm red[32], redp[2][3];
     pdl_wait();
@@ -498,7 +507,8 @@ __global__ void __launch_bounds__(MAXT, fx_k2_blocks(MAXT)) k2_fx(FxDev op, doub
 // --------------------------------------------------------------------- launch
 static Launch fx_rows_launch(const FxDev& v, int ept, int nb) {
     const int G = v.M1 / ept;
-    int TR = kFxTileRows;
+    // one row per block while that leaves no SM with two
+    int TR = (long)v.n2 * v.planes * nb <= 152 ? 1 : kFxTileRows;
     while (TR > 1 && TR * G > kRowsMaxThreads) TR /= 2;
     return Launch{dim3((v.n2 + TR - 1) / TR, v.planes, nb), dim3(TR * G), (size_t)TR * tile_stride(v.M1) * sizeof(fxc)};
 }

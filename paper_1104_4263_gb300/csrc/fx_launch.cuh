@@ -38,7 +38,7 @@ template <int EPT, int R0, int R1, int LS> struct FxLaunch {
                      cudaStream_t st, int nb);
 };
 
-template <int LS> using FxLaunch2 = FxLaunch<16, fx_plan(LS).r0, fx_plan(LS).r1, LS>;    // 2^a
+template <int LS> using FxLaunch2 = FxLaunch<fx_plan(LS).ept, fx_plan(LS).r0, fx_plan(LS).r1, LS>;    // 2^a
 template <int R0> using FxLaunch3 = FxLaunch<12, R0, 4, 0>;                              // 3 * 2^a
 
 }  // namespace die

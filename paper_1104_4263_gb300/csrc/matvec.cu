@@ -47,6 +47,12 @@ template <typename F> static void fx_for_length(int L, F&& f) {
         case 1024: f(FxLaunch2<1024>{}); return;
         case 2048: f(FxLaunch2<2048>{}); return;
         case 4096: f(FxLaunch2<4096>{}); return;
+        case 48: f(FxLaunch2<48>{}); return;
+        case 96: f(FxLaunch2<96>{}); return;
+        case 192: f(FxLaunch2<192>{}); return;
+        case 384: f(FxLaunch2<384>{}); return;
+        case 768: f(FxLaunch2<768>{}); return;
+        case 1536: f(FxLaunch2<1536>{}); return;
         default: break;
     }
     if (fx_plan(L).r0 == 6) f(FxLaunch3<6>{});
