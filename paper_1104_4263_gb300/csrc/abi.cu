@@ -11,6 +11,7 @@
 #include <tuple>
 #include <vector>
 
+#include "gx.cuh"
 #include "op.cuh"
 #include "solver.cuh"
 
@@ -77,7 +78,8 @@ int choose_fft_size(int n) {
     return best;
 }
 
-// Twiddle arrays (FP64: the natural table only; complex64: 3 L entries): [0, L) the natural table exp(-2 pi i m / L); for
+// Twiddle arrays (FP64: the natural table only; complex64: 4 L entries, the last L the
+// any-grid plan's, gx.cuh): [0, L) the natural table exp(-2 pi i m / L); for
 // L = 2^a in [256, 4096] (the compile-time stages of fft_fast.cuh), [L, 2 L) and
 // [2 L, 3 L) the stage tables of the forward and inverse plans: stage s (radix R,
 // sub-transform length Ns) keeps at r Ns + k - 1 (1 <= r < R, k < Ns) the natural entry
@@ -98,7 +100,7 @@ static void stage_table(int L, bool inv, const V* nat, V* out) {
 static void twiddles(int L, std::vector<double2>& d, std::vector<float2>& f, std::vector<fxw>& w) {
     d.assign((size_t)L, make_double2(0.0, 0.0));
     std::vector<fxw> nat(L);
-    f.assign(3 * (size_t)L, make_float2(0.f, 0.f));
+    f.assign(4 * (size_t)L, make_float2(0.f, 0.f));
     const long double two_pi = 6.283185307179586476925286766559005768L;
     for (int m = 0; m < L; m++) {
         const long double ang = two_pi * (long double)m / (long double)L;
@@ -111,12 +113,16 @@ static void twiddles(int L, std::vector<double2>& d, std::vector<float2>& f, std
     if (L >= 256 && L <= 4096 && (L & (L - 1)) == 0) {
         for (int inv = 0; inv < 2; inv++) stage_table(L, inv != 0, f.data(), f.data() + (1 + inv) * (size_t)L);
     }
-    // factors of the fixed-point plan (fx.cuh): stage (R, Ns) at r Ns + k - 1
+    // factors of the fixed-point (fx.cuh) and any-grid (gx.cuh) plans: stage (R, Ns) at
+    // r Ns + k - 1
     w.assign((size_t)L, fxw{0, 0, 0, 0});
-    const FxPlan p = fx_plan(L);
-    for (int s = 1, ns = p.r0; s <= p.q; ns *= p.r1, s++)
-        for (int r = 1; r < p.r1; r++)
-            for (int k = 0; k < ns; k++) w[r * ns + k - 1] = nat[(long)(L / (ns * p.r1)) * r * k];
+    auto fill = [L](const FxPlan& p, const auto* from, auto* to) {
+        for (int s = 1, ns = p.r0; s <= p.q; ns *= p.r1, s++)
+            for (int r = 1; r < p.r1; r++)
+                for (int k = 0; k < ns; k++) to[r * ns + k - 1] = from[(long)(L / (ns * p.r1)) * r * k];
+    };
+    fill(fx_plan(L), nat.data(), w.data());
+    fill(gx_plan(L), f.data(), f.data() + 3 * (size_t)L);
 }
 
 static std::atomic<uint64_t> g_next_id{1};
@@ -301,8 +307,8 @@ static die_status create_impl(const dieop_desc* desc, const void* eps_r, int eps
     DIE_TRY(dmalloc(&op->tw2_d, (size_t)op->M2 * sizeof(double2)));
     DIE_TRY(dmalloc(&op->fx1, (size_t)op->M1 * sizeof(fxw)));
     DIE_TRY(dmalloc(&op->fx2, (size_t)op->M2 * sizeof(fxw)));
-    DIE_TRY(dmalloc(&op->tw1_f, 3 * (size_t)op->M1 * sizeof(float2)));
-    DIE_TRY(dmalloc(&op->tw2_f, 3 * (size_t)op->M2 * sizeof(float2)));
+    DIE_TRY(dmalloc(&op->tw1_f, 4 * (size_t)op->M1 * sizeof(float2)));
+    DIE_TRY(dmalloc(&op->tw2_f, 4 * (size_t)op->M2 * sizeof(float2)));
     const int ng = green_plane_count(op);
     DIE_TRY(dmalloc(&op->gx, ng * q * sizeof(fxw)));
     DIE_TRY(dmalloc(&op->ge, op->Q1 * sizeof(int)));

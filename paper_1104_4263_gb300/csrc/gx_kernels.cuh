@@ -1,0 +1,276 @@
+// Product passes of the complex64 operators on any grid (n <= M / 2, M = 2^a or 3 * 2^a, two or
+// three planes): the passes K1, K2, K3 and K3K1 of matvec_kernels.cuh, same workspace layout.
+// Bound by latency: a pass is one wave of blocks on grids up to about 512^2.
+#pragma once
+
+#include "gx_launch.cuh"
+#include "matvec_kernels.cuh"
+
+namespace die {
+
+constexpr int kGxTileRows = 4;    // rows per block: 32-byte segments in the transposed accesses
+
+template <int EPT> __device__ __forceinline__ void gx_swap(float2 (&x)[EPT]) {
+#pragma unroll
+    for (int e = 0; e < EPT; e++) x[e] = make_float2(x[e].y, x[e].x);
+}
+
+// The transform of x (first-stage registers) into last-stage registers; buf: the transform's
+// part of shared memory, free to write.  All threads of the block call it.
+template <int LS> __device__ __forceinline__ void gx_transform(float2 (&x)[gx_plan(LS).ept], float2* buf,
+                                                               const float2* tw, int t) {
+    constexpr FxPlan p = gx_plan(LS);
+    constexpr int EPT = p.ept, R0 = p.r0, R1 = p.r1, G = LS / EPT;
+    gx_stage<EPT, R0>(x, 1, t, G, tw);
+    stage_store<float2, EPT, R0>(buf, x, LS, 1, t, G);
+    __syncthreads();
+    int Ns = R0;
+#pragma unroll
+    for (int s = 1; s <= p.q; s++) {
+        stage_load<float2, EPT, R1>(buf, x, LS, t, G);
+        gx_stage<EPT, R1>(x, Ns, t, G, tw);
+        __syncthreads();
+        if (s < p.q) {
+            stage_store<float2, EPT, R1>(buf, x, LS, Ns, t, G);
+            __syncthreads();
+        }
+        Ns *= R1;
+    }
+}
+
+// Rows of the tile to / from W[c][k1][row].
+__device__ __forceinline__ void gx_store_tile(const float2* tile, float2* __restrict__ W, int c, int i2_0, int L,
+                                              int n2, int TR, int Lp) {
+    const int sh = TR == 4 ? 2 : (TR == 2 ? 1 : 0);
+#pragma unroll 4
+    for (int e = threadIdx.x; e < L * TR; e += blockDim.x) {
+        const int k1 = e >> sh, r = e & (TR - 1);
+        if (i2_0 + r < n2) W[((long)c * L + k1) * n2 + i2_0 + r] = tile[r * Lp + pidx(k1)];
+    }
+}
+__device__ __forceinline__ void gx_load_tile(float2* tile, const float2* __restrict__ W, int c, int i2_0, int L, int n2,
+                                             int TR, int Lp) {
+    const int sh = TR == 4 ? 2 : (TR == 2 ? 1 : 0);
+#pragma unroll 8
+    for (int e = threadIdx.x; e < L * TR; e += blockDim.x) {
+        const int k1 = e >> sh, r = e & (TR - 1);
+        tile[r * Lp + pidx(k1)] = i2_0 + r < n2 ? W[((long)c * L + k1) * n2 + i2_0 + r] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+}
+
+// ------------------------------------------------------------------------- K1
+template <typename IO, int LS>
+__global__ void __launch_bounds__(512) k1_gx(OpDev<float> op, const IO* __restrict__ u, const float2* __restrict__ chi,
+                                             float2* __restrict__ W, const int* __restrict__ skip) {
+    constexpr FxPlan p = gx_plan(LS);
+    constexpr int EPT = p.ept, G = LS / EPT;
+    pdl_wait();
+    if (block_flag(skip)) return;
+    u += blockIdx.z * op.xs;            // right-hand side of a batched product
+    W += blockIdx.z * op.ws;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int TR = blockDim.x / G, Lp = tile_stride(LS);
+    const int rs = threadIdx.x / G, t = threadIdx.x - rs * G;
+    const int c = blockIdx.y, i2_0 = blockIdx.x * TR, i2 = i2_0 + rs;
+    const bool active = i2 < op.n2;
+    const IO* ur = u + c * ((long)op.n1 * op.n2) + (long)i2 * op.n1;
+    const float2* cr = (c == 2 ? op.chim : chi) + (long)i2 * op.n1;      // H3 plane: chi_m
+    float2* buf = reinterpret_cast<float2*>(smem_raw) + rs * Lp;
+    float2 x[EPT];
+#pragma unroll
+    for (int e = 0; e < EPT; e++) {
+        const int j = fx_slot<EPT, p.r0>(e), idx = t + j * G;
+        x[e] = j < EPT / 2 && active && idx < op.n1 ? cmul(cvt<float2>(ur[idx]), cr[idx]) : make_float2(0.f, 0.f);
+    }
+    gx_transform<LS>(x, buf, op.gx1, t);
+    stage_store<float2, EPT, p.r1>(buf, x, LS, LS / p.r1, t, G);
+    __syncthreads();
+    gx_store_tile(reinterpret_cast<const float2*>(smem_raw), W, c, i2_0, LS, op.n2, TR, Lp);
+}
+
+// ------------------------------------------------------------------------- K3
+template <typename U, typename IO, int LS>
+__global__ void __launch_bounds__(512) k3_gx(OpDev<float> op, const float2* __restrict__ W, const U* __restrict__ u,
+                                             IO* __restrict__ y, const int* __restrict__ skip) {
+    constexpr FxPlan p = gx_plan(LS);
+    constexpr int EPT = p.ept, G = LS / EPT;
+    pdl_wait();
+    if (block_flag(skip)) return;
+    W += blockIdx.z * op.ws;            // right-hand side of a batched product
+    u += blockIdx.z * op.xs;
+    y += blockIdx.z * op.xs;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int TR = blockDim.x / G, Lp = tile_stride(LS);
+    const int rs = threadIdx.x / G, t = threadIdx.x - rs * G;
+    const int c = blockIdx.y, i2_0 = blockIdx.x * TR, i2 = i2_0 + rs;
+    float2* buf = reinterpret_cast<float2*>(smem_raw) + rs * Lp;
+    gx_load_tile(reinterpret_cast<float2*>(smem_raw), W, c, i2_0, LS, op.n2, TR, Lp);
+    float2 x[EPT];
+    stage_load<float2, EPT, p.r0>(buf, x, LS, t, G);
+    gx_swap<EPT>(x);
+    __syncthreads();
+    gx_transform<LS>(x, buf, op.gx1, t);
+    if (i2 >= op.n2) return;
+    const long off = c * ((long)op.n1 * op.n2) + (long)i2 * op.n1;
+#pragma unroll
+    for (int e = 0; e < EPT; e++) {
+        const int j = fx_slot<EPT, p.r1>(e), idx = t + j * G;
+        if (j < EPT / 2 && idx < op.n1) y[off + idx] = csub(cvt<IO>(u[off + idx]), cvt<IO>(make_float2(x[e].y, x[e].x)));
+    }
+}
+
+// ----------------------------------------------------------------------- K3K1
+template <typename IO, int LS>
+__global__ void __launch_bounds__(512) k3k1_gx(OpDev<float> op, float2* __restrict__ W, const IO* __restrict__ u,
+                                               const float2* __restrict__ chir, float2* __restrict__ vbuf,
+                                               const int* __restrict__ skip) {
+    constexpr FxPlan p = gx_plan(LS);
+    constexpr int EPT = p.ept, G = LS / EPT;
+    pdl_wait();
+    if (block_flag(skip)) return;
+    W += blockIdx.z * op.ws;            // right-hand side of a batched product
+    u += blockIdx.z * op.xs;
+    vbuf += blockIdx.z * op.xs;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int TR = blockDim.x / G, Lp = tile_stride(LS);
+    const int rs = threadIdx.x / G, t = threadIdx.x - rs * G;
+    const int c = blockIdx.y, i2_0 = blockIdx.x * TR, i2 = i2_0 + rs;
+    const bool active = i2 < op.n2;
+    float2* buf = reinterpret_cast<float2*>(smem_raw) + rs * Lp;
+    gx_load_tile(reinterpret_cast<float2*>(smem_raw), W, c, i2_0, LS, op.n2, TR, Lp);
+    float2 x[EPT], z[EPT];
+    stage_load<float2, EPT, p.r0>(buf, x, LS, t, G);
+    gx_swap<EPT>(x);
+    __syncthreads();
+    gx_transform<LS>(x, buf, op.gx1, t);
+    // v = u - z (first product), kept for the final subtraction; then chi' v
+    const long off = c * ((long)op.n1 * op.n2) + (long)i2 * op.n1;
+    const float2* cr = (c == 2 ? op.chim : chir) + (long)i2 * op.n1;     // the regulariser keeps chi_m
+#pragma unroll
+    for (int e = 0; e < EPT; e++) {
+        const int j = fx_slot<EPT, p.r0>(e), idx = t + j * G, f = fx_reg<EPT, p.r1>(j);
+        z[e] = make_float2(0.f, 0.f);
+        if (j < EPT / 2 && active && idx < op.n1) {
+            const float2 v = csub(cvt<float2>(u[off + idx]), make_float2(x[f].y, x[f].x));
+            vbuf[off + idx] = v;
+            z[e] = cmul(v, cr[idx]);
+        }
+    }
+    gx_transform<LS>(z, buf, op.gx1, t);
+    stage_store<float2, EPT, p.r1>(buf, z, LS, LS / p.r1, t, G);
+    __syncthreads();
+    gx_store_tile(reinterpret_cast<const float2*>(smem_raw), W, c, i2_0, LS, op.n2, TR, Lp);
+}
+
+// ------------------------------------------------------------------------- K2
+// One block per column k1, G threads per plane; the Green multiply at the first inverse
+// stage's indices (planes G11, G22, G12 (G13, G23, G33), of parity -1 in both / x2 / x1 for
+// G12 / G13 / G23).
+template <int P, int LS>
+__global__ void __launch_bounds__(P * (LS / gx_plan(LS).ept)) k2_gx(OpDev<float> op, float2* __restrict__ W,
+                                                                 const int* __restrict__ skip) {
+    constexpr FxPlan p = gx_plan(LS);
+    constexpr int EPT = p.ept, G = LS / EPT, Q2 = LS / 2 + 1;
+    pdl_wait();
+    if (block_flag(skip)) return;
+    W += blockIdx.y * op.ws;            // right-hand side of a batched product
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int Lp = padded_len(LS);
+    float2* bufs = reinterpret_cast<float2*>(smem_raw);
+    const int comp = threadIdx.x / G, t = threadIdx.x - comp * G;
+    float2* buf = bufs + comp * Lp;
+    const int k1 = blockIdx.x;
+    float2* col = W + ((long)comp * op.M1 + k1) * op.n2;
+    const int h1 = op.M1 >> 1;
+    const int k1q = k1 <= h1 ? k1 : op.M1 - k1;
+    const bool neg1 = k1 > h1;
+    const long plane = (long)op.Q1 * Q2;
+    const float2* g = op.gq + (long)k1q * Q2;
+    float2 x[EPT];
+#pragma unroll
+    for (int e = 0; e < EPT; e++) {
+        const int j = fx_slot<EPT, p.r0>(e), idx = t + j * G;
+        x[e] = j < EPT / 2 && idx < op.n2 ? col[idx] : make_float2(0.f, 0.f);
+    }
+    gx_transform<LS>(x, buf, op.gx2, t);
+    stage_store<float2, EPT, p.r1>(buf, x, LS, LS / p.r1, t, G);
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < EPT; e++) {
+        const int k2 = t + fx_slot<EPT, p.r0>(e) * G;
+        const bool neg2 = k2 > LS / 2;
+        const int k2q = neg2 ? LS - k2 : k2;
+        float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < P; q++) {
+            const int pl = q == comp ? (q == 2 ? 5 : q) : (q + comp == 1 ? 2 : q + comp + 1);
+            const bool neg = q != comp && (q + comp == 1 ? neg1 != neg2 : (q + comp == 2 ? neg2 : neg1));
+            float2 w = __ldg(&g[pl * plane + k2q]);
+            if (neg) w = make_float2(-w.x, -w.y);
+            acc = cadd(acc, cmul(w, bufs[q * Lp + pidx(k2)]));
+        }
+        x[e] = make_float2(acc.y, acc.x);
+    }
+    __syncthreads();
+    gx_transform<LS>(x, buf, op.gx2, t);
+#pragma unroll
+    for (int e = 0; e < EPT; e++) {
+        const int j = fx_slot<EPT, p.r1>(e), idx = t + j * G;
+        if (j < EPT / 2 && idx < op.n2) col[idx] = make_float2(x[e].y, x[e].x);
+    }
+}
+
+// --------------------------------------------------------------------- launch
+template <int LS> static Launch gx_rows_launch(const OpDev<float>& v, int nb) {
+    constexpr int G = LS / gx_plan(LS).ept;
+    int TR = kGxTileRows;
+    // fewer rows per block while that leaves no SM with two blocks
+    while (TR > 1 && (TR * G > kRowsMaxThreads || (long)(2 * v.n2 / TR) * v.planes * nb <= 152)) TR /= 2;
+    return Launch{dim3((v.n2 + TR - 1) / TR, v.planes, nb), dim3(TR * G), (size_t)TR * tile_stride(LS) * sizeof(float2)};
+}
+template <int LS> template <typename IO>
+void GxLaunch<LS>::k1(const OpDev<float>& v, const IO* u, const float2* chi, float2* W, const int* skip,
+                      cudaStream_t st, int nb) {
+    static std::atomic<bool> a{false};
+    launch_kernel(k1_gx<IO, LS>, a, gx_rows_launch<LS>(v, nb), st, v, u, chi, W, skip);
+}
+template <int LS> template <typename U, typename IO>
+void GxLaunch<LS>::k3(const OpDev<float>& v, const float2* W, const U* u, IO* y, const int* skip, cudaStream_t st, int nb) {
+    static std::atomic<bool> a{false};
+    launch_kernel(k3_gx<U, IO, LS>, a, gx_rows_launch<LS>(v, nb), st, v, W, u, y, skip);
+}
+template <int LS> template <typename IO>
+void GxLaunch<LS>::k3k1(const OpDev<float>& v, float2* W, const IO* u, const float2* chir, float2* vb, const int* skip,
+                        cudaStream_t st, int nb) {
+    static std::atomic<bool> a{false};
+    launch_kernel(k3k1_gx<IO, LS>, a, gx_rows_launch<LS>(v, nb), st, v, W, u, chir, vb, skip);
+}
+template <int LS>
+void GxLaunch<LS>::k2(const OpDev<float>& v, float2* W, const int* skip, cudaStream_t st, int nb) {
+    static std::atomic<bool> a2{false}, a3{false};
+    const Launch l{dim3(v.M1, nb), dim3(v.planes * (LS / gx_plan(LS).ept)),
+                   (size_t)v.planes * padded_len(LS) * sizeof(float2)};
+    if (v.planes == 3) launch_kernel(k2_gx<3, LS>, a3, l, st, v, W, skip);
+    else launch_kernel(k2_gx<2, LS>, a2, l, st, v, W, skip);
+}
+
+// Instantiates the launchers of one length.
+#define DIE_GX_INSTANTIATE(LS)                                                                                       \
+    template void GxLaunch<LS>::k1<float2>(const OpDev<float>&, const float2*, const float2*, float2*, const int*,   \
+                                           cudaStream_t, int);                                                      \
+    template void GxLaunch<LS>::k1<double2>(const OpDev<float>&, const double2*, const float2*, float2*, const int*, \
+                                            cudaStream_t, int);                                                     \
+    template void GxLaunch<LS>::k2(const OpDev<float>&, float2*, const int*, cudaStream_t, int);                     \
+    template void GxLaunch<LS>::k3<float2, float2>(const OpDev<float>&, const float2*, const float2*, float2*,       \
+                                                   const int*, cudaStream_t, int);                                  \
+    template void GxLaunch<LS>::k3<double2, double2>(const OpDev<float>&, const float2*, const double2*, double2*,   \
+                                                     const int*, cudaStream_t, int);                                \
+    template void GxLaunch<LS>::k3<float2, double2>(const OpDev<float>&, const float2*, const float2*, double2*,     \
+                                                    const int*, cudaStream_t, int);                                 \
+    template void GxLaunch<LS>::k3k1<float2>(const OpDev<float>&, float2*, const float2*, const float2*, float2*,    \
+                                             const int*, cudaStream_t, int);                                        \
+    template void GxLaunch<LS>::k3k1<double2>(const OpDev<float>&, float2*, const double2*, const float2*, float2*,  \
+                                              const int*, cudaStream_t, int);
+
+}  // namespace die

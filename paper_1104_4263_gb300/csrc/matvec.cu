@@ -27,6 +27,7 @@ OpDev<float> view_f(const dieop_s* op) {
     v.ws = (long)op->planes * op->M1 * op->n2;
     v.tw1 = op->tw1_f; v.tw2 = op->tw2_f; v.gq = op->gq_f;
     v.twx1 = op->tw1_f + op->M1; v.twx2 = op->tw2_f + op->M2;
+    v.gx1 = op->tw1_f + 3 * (size_t)op->M1; v.gx2 = op->tw2_f + 3 * (size_t)op->M2;
     v.tr = op->tile_rows_c64;
     v.chim = op->chim_f;
     return v;

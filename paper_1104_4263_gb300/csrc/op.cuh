@@ -16,6 +16,7 @@ struct OpDev {
     const C* tw2;                 // exp(-2 pi i m / M2)
     const C* twx1;                // stage tables of the compile-time plans along x1 (2 M1)
     const C* twx2;                // the same along x2 (2 M2)
+    const float2 *gx1, *gx2;      // factors of the any-grid plans (gx.cuh) along x1 and x2
     const C* gq;                  // quarter spectra of G11, G22, G12 (and, with three planes, G13,
                                   // G23, G33): [plane][k1q][k2q], pre-scaled
     const C* chim;                // magnetic contrast chi_m (three planes; null otherwise)
@@ -56,8 +57,8 @@ struct dieop_s {
     die_polarization pol = DIE_TE;
     die::FftPlan f1{}, i1{}, f2{}, i2{};
     double2 *tw1_d = nullptr, *tw2_d = nullptr;   // M entries: natural table (set-up only)
-    float2 *tw1_f = nullptr, *tw2_f = nullptr;    // 3 M entries: natural table, then the
-                                                  // forward and inverse stage tables
+    float2 *tw1_f = nullptr, *tw2_f = nullptr;    // 4 M entries: natural table, the forward and
+                                                  // inverse stage tables, the any-grid plan's
     die::fxw *fx1 = nullptr, *fx2 = nullptr;      // M entries: factors of the fixed-point plans
     int planes = 2;                // field planes: 3 for DIE_TE_MAG (E1, E2, H3)
     die::fxw* gx = nullptr;        // (planes == 3 ? 6 : 3) * Q1 * Q2, fixed point, one scale
