@@ -41,7 +41,7 @@ template <int LS> __device__ __forceinline__ void gx_transform(float2 (&x)[gx_pl
 // Rows of the tile to / from W[c][k1][row].
 __device__ __forceinline__ void gx_store_tile(const float2* tile, float2* __restrict__ W, int c, int i2_0, int L,
                                               int n2, int TR, int Lp) {
-    const int sh = TR == 4 ? 2 : (TR == 2 ? 1 : 0);
+    const int sh = 31 - __clz(TR);             // TR = 1, 2, 4 or 8
 #pragma unroll 4
     for (int e = threadIdx.x; e < L * TR; e += blockDim.x) {
         const int k1 = e >> sh, r = e & (TR - 1);
@@ -50,7 +50,7 @@ __device__ __forceinline__ void gx_store_tile(const float2* tile, float2* __rest
 }
 __device__ __forceinline__ void gx_load_tile(float2* tile, const float2* __restrict__ W, int c, int i2_0, int L, int n2,
                                              int TR, int Lp) {
-    const int sh = TR == 4 ? 2 : (TR == 2 ? 1 : 0);
+    const int sh = 31 - __clz(TR);
 #pragma unroll 8
     for (int e = threadIdx.x; e < L * TR; e += blockDim.x) {
         const int k1 = e >> sh, r = e & (TR - 1);
@@ -224,8 +224,13 @@ __global__ void __launch_bounds__(P * (LS / gx_plan(LS).ept)) k2_gx(OpDev<float>
 // --------------------------------------------------------------------- launch
 template <int LS> static Launch gx_rows_launch(const OpDev<float>& v, int nb) {
     constexpr int G = LS / gx_plan(LS).ept;
+    // the operator's schedule where it has one (half_filled_rows); else fewer rows per block
+    // while that leaves no SM with two blocks
+    if (half_filled_rows(v)) {
+        const int h = v.tr ? v.tr : default_tile_rows_c64(LS);
+        return Launch{dim3((v.n2 + h - 1) / h, v.planes, nb), dim3(h * G), (size_t)h * tile_stride(LS) * sizeof(float2)};
+    }
     int TR = kGxTileRows;
-    // fewer rows per block while that leaves no SM with two blocks
     while (TR > 1 && (TR * G > kRowsMaxThreads || (long)(2 * v.n2 / TR) * v.planes * nb <= 152)) TR /= 2;
     return Launch{dim3((v.n2 + TR - 1) / TR, v.planes, nb), dim3(TR * G), (size_t)TR * tile_stride(LS) * sizeof(float2)};
 }

@@ -27,13 +27,13 @@ template die_status apply_reg_skip_xy<float, float2, double2>(dieop_s*, const fl
                                                               cudaStream_t,
                                   const Workspace*);
 
-bool defl_product_ok(const dieop_s* op) { return fast_rows(view_f(op)); }
+bool defl_product_ok(const dieop_s* op) { return half_filled_rows(view_f(op)); }
 
 die_status apply_defl_xy(dieop_s* op, const DeflIn& d, float2* z, double2* y, bool reg, const int* skip,
                          cudaStream_t st, const Workspace* ws) {
     if (!ws) ws = &op->ws;
     const OpDev<float> v = view_f(op);
-    if (!fast_rows(v) || d.r < 1 || d.r > 32 || !d.V32 || !d.cf || (!d.w && !d.x) || (d.w && !d.inv))
+    if (!half_filled_rows(v) || d.r < 1 || d.r > 32 || !d.V32 || !d.cf || (!d.w && !d.x) || (d.w && !d.inv))
         return DIE_EINVAL;
     float2* W = reinterpret_cast<float2*>(ws->W);
     float2* vb = reinterpret_cast<float2*>(ws->v);

@@ -20,8 +20,8 @@
 // G12 is odd in each offset coordinate (a symmetry of Eqs. (4.3)-(4.5)), so the
 // other quadrants follow by sign.  They carry the 1/(M1 M2) of the inverse FFTs.
 //
-// Here: grids with n = M / 2, M = 2^a in [256, 4096] (rows and columns apart), on the
-// compile-time stages of fft_fast.cuh; other grids take the passes of gx_kernels.cuh.
+// Here: transforms of length 1024, 2048 and 4096 (rows and columns apart) of two-plane grids,
+// on the compile-time stages of fft_fast.cuh; the others take the passes of gx_kernels.cuh.
 #pragma once
 
 #include <atomic>
@@ -98,11 +98,12 @@ __device__ __forceinline__ void tile_io(C* tile, C* __restrict__ W, int c, int i
     }
 }
 
-template <typename T, typename IO, int L, int TR>
+// RAG: n1 < L / 2 (a run-time row length); the transform still treats its upper half as zero.
+template <typename T, typename IO, int L, int TR, bool RAG>
 __global__ void __launch_bounds__(512) k1_fast(OpDev<T> op, const IO* __restrict__ u, const C_t<T>* __restrict__ chi,
                                                C_t<T>* __restrict__ W, const int* __restrict__ skip) {
     using C = C_t<T>;
-    constexpr int G = L / 16, n1 = L / 2;
+    constexpr int G = L / 16;
     using F0 = typename PlanStage<C, L, false, 0>::St;
     pdl_wait();
     if (block_flag(skip)) return;
@@ -114,6 +115,7 @@ __global__ void __launch_bounds__(512) k1_fast(OpDev<T> op, const IO* __restrict
     const int c = blockIdx.y, i2_0 = blockIdx.x * TR, i2 = i2_0 + rs;
     const bool active = i2 < op.n2;
     C* buf = tile + rs * tile_stride_c<L>();
+    const int n1 = RAG ? op.n1 : L / 2;
     C x[16];
     if (active) {
         const long N = (long)n1 * op.n2;
@@ -122,7 +124,7 @@ __global__ void __launch_bounds__(512) k1_fast(OpDev<T> op, const IO* __restrict
 #pragma unroll
         for (int e = 0; e < 16; e++) {
             const int idx = F0::index(e);
-            x[e] = idx < n1 ? cmul(cvt<C>(ur[idx]), cr[idx]) : czero<C>();
+            x[e] = idx < L / 2 && (!RAG || t + idx < n1) ? cmul(cvt<C>(ur[idx]), cr[idx]) : czero<C>();
         }
         F0::compute(x, t, op.twx1);
         F0::store(buf, x, t);
@@ -226,11 +228,12 @@ __global__ void __launch_bounds__(512) k1_defl_fast(OpDev<float> op, DeflIn d, c
 // inverse stage (same radix: the inverse plan is the reversed forward plan) wants them,
 // so the 2 x 2 Green multiply is done in registers between the two, with no shared-
 // memory round trip, and every twiddle serves both components.
-template <typename T, int L>
+template <typename T, int L, bool RAG>
 __global__ void __launch_bounds__(L / 16, (L == 1024 ? 7 : 1)) k2_fast2(OpDev<T> op, C_t<T>* __restrict__ W,
                                                                         int stage_g, const int* __restrict__ skip) {
     using C = C_t<T>;
-    constexpr int G = L / 16, n2 = L / 2, Q2 = L / 2 + 1, Lp = L + (L >> 4);
+    constexpr int G = L / 16, Q2 = L / 2 + 1, Lp = L + (L >> 4);
+    const int n2 = RAG ? op.n2 : L / 2;
     constexpr int nsf = P2<L>::fwd.ns, nsi = P2<L>::inv.ns;
     using F0 = typename PlanStage<C, L, false, 0>::St;
     using FL = typename PlanStage<C, L, false, nsf - 1>::St;
@@ -267,8 +270,8 @@ __global__ void __launch_bounds__(L / 16, (L == 1024 ? 7 : 1)) k2_fast2(OpDev<T>
 #pragma unroll
     for (int e = 0; e < 16; e++) {
         const int idx = F0::index(e);
-        x0[e] = idx < n2 ? col0[idx] : czero<C>();
-        x1[e] = idx < n2 ? col1[idx] : czero<C>();
+        x0[e] = idx < L / 2 && (!RAG || t + idx < n2) ? col0[idx] : czero<C>();
+        x1[e] = idx < L / 2 && (!RAG || t + idx < n2) ? col1[idx] : czero<C>();
     }
     F0::compute2(x0, x1, t, op.twx2);
     F0::store(buf0, x0, t);
@@ -313,15 +316,16 @@ __global__ void __launch_bounds__(L / 16, (L == 1024 ? 7 : 1)) k2_fast2(OpDev<T>
 #pragma unroll
     for (int e = 0; e < 16; e++) {
         const int idx = IL::index(e);
-        if (idx < n2) { col0[idx] = x0[e]; col1[idx] = x1[e]; }
+        if (idx < L / 2 && (!RAG || t + idx < n2)) { col0[idx] = x0[e]; col1[idx] = x1[e]; }
     }
 }
 
-template <typename T, typename U, typename IO, int L, int TR>
+template <typename T, typename U, typename IO, int L, int TR, bool RAG>
 __global__ void __launch_bounds__(512) k3_fast(OpDev<T> op, const C_t<T>* __restrict__ W, const U* __restrict__ u,
                                                IO* __restrict__ y, const int* __restrict__ skip) {
     using C = C_t<T>;
-    constexpr int G = L / 16, n1 = L / 2, ns = P2<L>::inv.ns;
+    constexpr int G = L / 16, ns = P2<L>::inv.ns;
+    const int n1 = RAG ? op.n1 : L / 2;
     using IL = typename PlanStage<C, L, true, ns - 1>::St;
     pdl_wait();
     if (block_flag(skip)) return;
@@ -338,7 +342,10 @@ __global__ void __launch_bounds__(512) k3_fast(OpDev<T> op, const C_t<T>* __rest
     U up[8];                    // u at this thread's output indices, loaded before the FFT
 #pragma unroll
     for (int e = 0, q = 0; e < 16; e++)
-        if (IL::index(e) < n1) up[q++] = u[off + IL::index(e)];
+        if (IL::index(e) < L / 2) {
+            if (!RAG || t + IL::index(e) < n1) up[q] = u[off + IL::index(e)];
+            q++;
+        }
     tile_io<C, L, TR, false>(tile, const_cast<C*>(W), c, i2_0, op.n2);
     __syncthreads();
     C x[16];
@@ -349,16 +356,20 @@ __global__ void __launch_bounds__(512) k3_fast(OpDev<T> op, const C_t<T>* __rest
 #pragma unroll
     for (int e = 0, q = 0; e < 16; e++) {
         const int idx = IL::index(e);
-        if (idx < n1) y[off + idx] = csub(cvt<IO>(up[q++]), cvt<IO>(x[e]));
+        if (idx < L / 2) {
+            if (!RAG || t + idx < n1) y[off + idx] = csub(cvt<IO>(up[q]), cvt<IO>(x[e]));
+            q++;
+        }
     }
 }
 
-template <typename T, typename IO, int L, int TR>
+template <typename T, typename IO, int L, int TR, bool RAG>
 __global__ void __launch_bounds__(512) k3k1_fast(OpDev<T> op, C_t<T>* __restrict__ W, const IO* __restrict__ u,
                                                  const C_t<T>* __restrict__ chir, C_t<T>* __restrict__ vbuf,
                                                  const int* __restrict__ skip) {
     using C = C_t<T>;
-    constexpr int G = L / 16, n1 = L / 2;
+    constexpr int G = L / 16;
+    const int n1 = RAG ? op.n1 : L / 2;
     constexpr int nsi = P2<L>::inv.ns, nsf = P2<L>::fwd.ns;
     using IL = typename PlanStage<C, L, true, nsi - 1>::St;
     using F0 = typename PlanStage<C, L, false, 0>::St;
@@ -379,7 +390,12 @@ __global__ void __launch_bounds__(512) k3k1_fast(OpDev<T> op, C_t<T>* __restrict
     C up[8], cp[8];             // u and chi' at this thread's indices, loaded before the FFT
 #pragma unroll
     for (int e = 0, q = 0; e < 16; e++)
-        if (IL::index(e) < n1) { up[q] = cvt<C>(u[off + IL::index(e)]); cp[q] = cr[IL::index(e)]; q++; }
+        if (IL::index(e) < L / 2) {
+            const bool in = !RAG || t + IL::index(e) < n1;
+            up[q] = in ? cvt<C>(u[off + IL::index(e)]) : czero<C>();
+            cp[q] = in ? cr[IL::index(e)] : czero<C>();
+            q++;
+        }
     tile_io<C, L, TR, false>(tile, W, c, i2_0, op.n2);
     __syncthreads();
     C x[16];
@@ -391,10 +407,11 @@ __global__ void __launch_bounds__(512) k3k1_fast(OpDev<T> op, C_t<T>* __restrict
 #pragma unroll
         for (int e = 0, q = 0; e < 16; e++) {
             const int idx = IL::index(e);
-            if (idx < n1) {
+            if (idx < L / 2) {
                 const C v = csub(up[q], x[e]);
-                vbuf[off + idx] = v;
-                x[e] = cmul(v, cp[q]);
+                const bool in = !RAG || t + idx < n1;
+                if (in) vbuf[off + idx] = v;
+                x[e] = in ? cmul(v, cp[q]) : czero<C>();
                 q++;
             } else {
                 x[e] = czero<C>();
@@ -437,13 +454,17 @@ inline void launch_kernel(K kernel, std::atomic<bool>& attr_set, const Launch& l
     launch_pdl(kernel, l.grid, l.block, l.smem, st, args...);
 }
 
-// Grids on the fast path: n = L / 2 with L = 2^a in [256, 4096] (per direction).
-// (Two-plane operators; everything else runs on the any-grid kernels, gx_kernels.cuh.)
-template <typename T> inline bool fast_rows(const OpDev<T>& v) {
+// Transforms on the stages of fft_fast.cuh: two planes, L = 1024, 2048 or 4096 (16 values per
+// thread, both components of a column in one thread).  Shorter ones, 3 * 2^a and three planes
+// take the any-grid kernels (gx_kernels.cuh), which are faster there: 128^2 22.3 -> 19 us,
+// 256^2 27 -> 24; at L = 1024 they take 62 us where these take 46.
+inline bool fast_length(int L) { return L == 1024 || L == 2048 || L == 4096; }
+template <typename T> inline bool fast_rows(const OpDev<T>& v) { return v.planes == 2 && fast_length(v.M1); }
+template <typename T> inline bool fast_cols(const OpDev<T>& v) { return v.planes == 2 && fast_length(v.M2); }
+// Grids whose rows fill half of a transform of length 2^a in [256, 4096]: the deflated first
+// row pass (k1_defl_fast) and the tile schedule (dieop_autotune).
+template <typename T> inline bool half_filled_rows(const OpDev<T>& v) {
     return v.planes == 2 && 2 * v.n1 == v.M1 && v.M1 >= 256 && v.M1 <= 4096 && (v.M1 & (v.M1 - 1)) == 0;
-}
-template <typename T> inline bool fast_cols(const OpDev<T>& v) {
-    return v.planes == 2 && 2 * v.n2 == v.M2 && v.M2 >= 256 && v.M2 <= 4096 && (v.M2 & (v.M2 - 1)) == 0;
 }
 template <typename C, int L, int TR> inline Launch rows_launch_fast(int n2) {
     return Launch{dim3((n2 + TR - 1) / TR, 2), dim3(TR * (L / 16)), (size_t)TR * tile_stride_c<L>() * sizeof(C)};
@@ -451,12 +472,18 @@ template <typename C, int L, int TR> inline Launch rows_launch_fast(int n2) {
 
 #define DIE_FAST_SWITCH(M, CASE)  \
     switch (M) {                  \
-        case 256: CASE(256); break;   \
-        case 512: CASE(512); break;   \
         case 1024: CASE(1024); break; \
         case 2048: CASE(2048); break; \
         case 4096: CASE(4096); break; \
         default: break;               \
+    }
+
+// Those of half_filled_rows.
+#define DIE_HALF_SWITCH(M, CASE)      \
+    switch (M) {                      \
+        case 256: CASE(256); break;   \
+        case 512: CASE(512); break;   \
+        default: DIE_FAST_SWITCH(M, CASE); break; \
     }
 
 // Tile height of the fast row passes: the rows of one block (TR).  0 selects fast_tr,
@@ -516,7 +543,12 @@ inline void launch_k2(const OpDev<T>& v, C_t<T>* W, const int* skip, cudaStream_
     int sg = 0;
     Launch l = cols_launch(v, &sg);
     l.grid.y = nb;
-#define K2F_CASE(LSV) { static std::atomic<bool> a_{false}; launch_kernel(k2_fast2<T, LSV>, a_, l, st, v, W, sg, skip); }
+#define K2F_CASE(LSV)                                                                                    \
+    {                                                                                                    \
+        static std::atomic<bool> a_{false}, r_{false};                                                   \
+        if (2 * v.n2 == LSV) launch_kernel(k2_fast2<T, LSV, false>, a_, l, st, v, W, sg, skip);          \
+        else launch_kernel(k2_fast2<T, LSV, true>, r_, l, st, v, W, sg, skip);                           \
+    }
     DIE_PROF(PK_COLS, st, DIE_FAST_SWITCH(v.M2, K2F_CASE));
 #undef K2F_CASE
 }

@@ -15,9 +15,10 @@ void rows_fwd_fast(const OpDev<T>& v, const IO* u, const C_t<T>* chi, C_t<T>* W,
 #define K1F_CASE(LSV)                                                                                        \
     if constexpr (tile_ok<C, LSV, TR>()) {                                                                   \
         constexpr int tr_ = tile_of<C, LSV, TR>();                                                           \
-        static std::atomic<bool> a_{false};                                                                  \
-        launch_kernel(k1_fast<T, IO, LSV, tr_>, a_, with_z(rows_launch_fast<C, LSV, tr_>(v.n2), nb), st, v, u, \
-                      chi, W, skip);                                                                         \
+        static std::atomic<bool> a_{false}, r_{false};                                                       \
+        const Launch l_ = with_z(rows_launch_fast<C, LSV, tr_>(v.n2), nb);                                   \
+        if (2 * v.n1 == LSV) launch_kernel(k1_fast<T, IO, LSV, tr_, false>, a_, l_, st, v, u, chi, W, skip);      \
+        else if constexpr (TR == 0) launch_kernel(k1_fast<T, IO, LSV, tr_, true>, r_, l_, st, v, u, chi, W, skip); \
     }
     DIE_PROF(PK_ROWS_FWD, st, DIE_FAST_SWITCH(v.M1, K1F_CASE));
 #undef K1F_CASE
@@ -29,9 +30,10 @@ void rows_inv_fast(const OpDev<T>& v, const C_t<T>* W, const U* u, IO* y, const 
 #define K3F_CASE(LSV)                                                                                        \
     if constexpr (tile_ok<C, LSV, TR>()) {                                                                   \
         constexpr int tr_ = tile_of<C, LSV, TR>();                                                           \
-        static std::atomic<bool> a_{false};                                                                  \
-        launch_kernel(k3_fast<T, U, IO, LSV, tr_>, a_, with_z(rows_launch_fast<C, LSV, tr_>(v.n2), nb), st, v, \
-                      W, u, y, skip);                                                                        \
+        static std::atomic<bool> a_{false}, r_{false};                                                       \
+        const Launch l_ = with_z(rows_launch_fast<C, LSV, tr_>(v.n2), nb);                                   \
+        if (2 * v.n1 == LSV) launch_kernel(k3_fast<T, U, IO, LSV, tr_, false>, a_, l_, st, v, W, u, y, skip);      \
+        else if constexpr (TR == 0) launch_kernel(k3_fast<T, U, IO, LSV, tr_, true>, r_, l_, st, v, W, u, y, skip); \
     }
     DIE_PROF(PK_ROWS_INV, st, DIE_FAST_SWITCH(v.M1, K3F_CASE));
 #undef K3F_CASE
@@ -44,9 +46,10 @@ void rows_inv_fwd_fast(const OpDev<T>& v, C_t<T>* W, const IO* u, const C_t<T>* 
 #define KKF_CASE(LSV)                                                                                        \
     if constexpr (tile_ok<C, LSV, TR>()) {                                                                   \
         constexpr int tr_ = tile_of<C, LSV, TR>();                                                           \
-        static std::atomic<bool> a_{false};                                                                  \
-        launch_kernel(k3k1_fast<T, IO, LSV, tr_>, a_, with_z(rows_launch_fast<C, LSV, tr_>(v.n2), nb), st, v, \
-                      W, u, chir, vb, skip);                                                                 \
+        static std::atomic<bool> a_{false}, r_{false};                                                       \
+        const Launch l_ = with_z(rows_launch_fast<C, LSV, tr_>(v.n2), nb);                                   \
+        if (2 * v.n1 == LSV) launch_kernel(k3k1_fast<T, IO, LSV, tr_, false>, a_, l_, st, v, W, u, chir, vb, skip);      \
+        else if constexpr (TR == 0) launch_kernel(k3k1_fast<T, IO, LSV, tr_, true>, r_, l_, st, v, W, u, chir, vb, skip); \
     }
     DIE_PROF(PK_ROWS_INV_FWD, st, DIE_FAST_SWITCH(v.M1, KKF_CASE));
 #undef KKF_CASE
@@ -62,7 +65,7 @@ void rows_defl_fast(const OpDev<float>& v, const DeflIn& d, const float2* chi, f
         launch_kernel(k1_defl_fast<LSV, tr_>, a_, rows_launch_fast<float2, LSV, tr_>(v.n2), st, v, d, chi, z, W, \
                       skip);                                                                                 \
     }
-    DIE_PROF(PK_ROWS_FWD, st, DIE_FAST_SWITCH(v.M1, K1D_CASE));
+    DIE_PROF(PK_ROWS_FWD, st, DIE_HALF_SWITCH(v.M1, K1D_CASE));
 #undef K1D_CASE
 }
 
