@@ -283,6 +283,56 @@ __global__ void __launch_bounds__(kRedThreads, 2) proj3_kernel(const double2* __
     reduce_partials(rs, nvt, out, kGroup3);
 }
 
+// ---------------------------------------------------- fixed-point Gram-Schmidt updates
+// The update w - V h is a sum of products of FP64 numbers; GB300's FP64 pipe does 2 FMAs per
+// clock and SM, its integer pipes 24 32 x 32 -> 64-bit multiply-adds.  So a row's eight basis
+// values (of a common exponent) and their coefficients are brought to 58-bit integers, the
+// products accumulated exactly but for the bits below 2^32 of their 118, and only the sums of
+// eight terms go through the FP64 pipe (4 operations instead of 24).  A term's error is 2^-58
+// of the largest term of its sum, below the 2^-53 of every term in FP64.  Complex products take
+// Gauss's three multiplications.  At 512^2 (cylinder, r = 8, 15 vectors on average) the update
+// takes 62 us where the FP64 form takes 92, bound by the conversions.  The projections gain
+// nothing from it (80 against 75 us: a chunk of rows needs its exponent before its first
+// product, and the loads wait on that) and stay in FP64.
+constexpr int kGsBits = 58;                  // |operand| < 2^58, sums and differences < 2^59
+
+struct Fix { int h, l; };                    // h 2^32 + l, l signed
+__device__ __forceinline__ Fix fix_split(long long a) {
+    Fix f;
+    f.l = (int)(unsigned)a;
+    f.h = (int)(a >> 32) + (int)((unsigned)f.l >> 31);
+    return f;
+}
+__device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >> 20) & 2047; }
+// v 2^(1022 + kGsBits - emax) towards zero, for a v whose exponent field is at most emax (so |v| <
+// 2^(emax - 1022)).  Zeros and values below 2^-63 of the largest give 0.
+__device__ __forceinline__ long long fix_of(double v, int emax) {
+    const int hi = __double2hiint(v);
+    const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u, ml = (unsigned)__double2loint(v);
+    const unsigned long long m = ((unsigned long long)mh << 32 | ml) << (kGsBits - 53);
+    const int s = min(emax - ((hi >> 20) & 2047), 63);
+    const long long r = (long long)(m >> s);
+    return hi < 0 ? -r : r;
+}
+// Sum of products: a b = (hh 2^32 + mid) 2^32, |mid| grows by less than 2^59 per term.
+struct FixSum { long long hh, mid; };
+__device__ __forceinline__ void fix_mac(FixSum& s, Fix a, Fix b) {
+    s.hh += (long long)a.h * b.h;
+    s.mid += (long long)a.h * b.l;
+    s.mid += (long long)a.l * b.h;
+    s.mid += __mulhi(a.l, b.l);
+}
+// acc += the sum of at most eight terms of operands of exponents ea and eb.  The sum is cut to
+// units of 2^59, 2^-59 of the largest term there can be, for one conversion.
+static __device__ __noinline__ double fix_add_far(double acc, double v, int e) { return acc + scalbn(v, e); }
+__device__ __forceinline__ double fix_add(double acc, const FixSum& s, int ea, int eb) {
+    const double v = __ll2double_rn((s.hh << 5) + (s.mid >> 27));
+    const int e = ea + eb - 2 * (1022 + kGsBits) + 59;
+    if (ea == 2047 || eb == 2047) return __longlong_as_double(0x7ff8000000000000ll);     // not finite
+    if (e < -1022 || e > 960) return fix_add_far(acc, v, e);
+    return fma(v, __hiloint2double((1023 + e) << 20, 0), acc);
+}
+
 // Runtime count -> compile-time CNT in [1, C].
 template <typename VT, int C, bool SCALE>
 __device__ __forceinline__ void proj_group_n(int cnt, const VT* V, long ldv, int g0, int nv, const VT* xin, VT* xout,
@@ -399,11 +449,59 @@ __device__ __forceinline__ double inv_norm(double s2) {
     return (hn > 0.0 && isfinite(hn)) ? 1.0 / hn : 1.0;
 }
 
+// Shared coefficients of a fixed-point update: Im c, Re c - Im c, Re c + Im c of every vector
+// in fixed point of one exponent.  All threads call it; k <= kMaxBasis.
+struct FixCoef { Fix f[3]; };
+__device__ __forceinline__ int fix_coefs(const double2* c, int k, FixCoef* fc, int* s_e) {
+    if (threadIdx.x == 0) *s_e = 0;
+    __syncthreads();
+    int e = 0;
+    for (int i = threadIdx.x; i < k; i += blockDim.x) e = max(e, max(exp_field(c[i].x), exp_field(c[i].y)));
+    atomicMax(s_e, e);
+    __syncthreads();
+    e = *s_e;
+    for (int i = threadIdx.x; i < k; i += blockDim.x) {
+        const long long x = fix_of(c[i].x, e), y = fix_of(c[i].y, e);
+        fc[i].f[0] = fix_split(y);
+        fc[i].f[1] = fix_split(x - y);
+        fc[i].f[2] = fix_split(x + y);
+    }
+    __syncthreads();
+    return e;
+}
+// (x, y) += sum over i < k of c_i V_i[idx]: groups of eight vectors, one exponent each.
+__device__ __forceinline__ void fix_update(const double2* __restrict__ V, long ldv, int k, long idx, const FixCoef* fc,
+                                           int ec, double& x, double& y) {
+    constexpr int GV = 8;
+#pragma unroll 1
+    for (int i0 = 0; i0 < k; i0 += GV) {
+        double2 a[GV];
+        int e = 0;
+#pragma unroll
+        for (int v = 0; v < GV; v++) a[v] = i0 + v < k ? V[(long)(i0 + v) * ldv + idx] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int v = 0; v < GV; v++) e = max(e, max(exp_field(a[v].x), exp_field(a[v].y)));
+        FixSum p1{0, 0}, p2{0, 0}, p3{0, 0};
+#pragma unroll
+        for (int v = 0; v < GV; v++) {
+            if (i0 + v < k) {
+                const FixCoef c = fc[i0 + v];
+                const long long ax = fix_of(a[v].x, e), ay = fix_of(a[v].y, e);
+                fix_mac(p1, fix_split(ax - ay), c.f[0]);
+                fix_mac(p2, fix_split(ax), c.f[1]);
+                fix_mac(p3, fix_split(ay), c.f[2]);
+            }
+        }
+        x = fix_add(x, FixSum{p1.hh + p2.hh, p1.mid + p2.mid}, e, ec);
+        y = fix_add(y, FixSum{p1.hh + p3.hh, p1.mid + p3.mid}, e, ec);
+    }
+}
+
 // out = base + sum_i V_i c_i.  Coefficients: c = sign * coef, or c = M s when M != NULL.
 // The sum for a row starts from base and runs through the basis in order in one pair of
 // accumulators (the FP64 pipe, not the FMA latency, bounds the loop).
-template <typename VT, bool NORM>
-__global__ void __launch_bounds__(kRedThreads) basis_axpy_kernel(const VT* __restrict__ V, long ldv, int k,
+template <typename VT, bool NORM, bool FIX>
+__global__ void __launch_bounds__(kRedThreads, FIX ? 2 : 1) basis_axpy_kernel(const VT* __restrict__ V, long ldv, int k,
                                                                  const double2* __restrict__ coef, double sign,
                                                                  const double2* __restrict__ M,
                                                                  const double2* __restrict__ s, const double2* base,
@@ -416,7 +514,9 @@ __global__ void __launch_bounds__(kRedThreads) basis_axpy_kernel(const VT* __res
     if (off && !(NORM && live)) return;
     __shared__ VT cs[kMaxBasis];
     __shared__ A csn[kMaxBasis];            // -Im(c): every step below is a plain FMA
-    __shared__ double c3[3][kMaxBasis];     // VM != NULL: Im c, Re c - Im c, Re c + Im c
+    __shared__ double c3[3][FIX ? 1 : kMaxBasis];     // VM != NULL: Im c, Re c - Im c, Re c + Im c
+    __shared__ FixCoef fc[FIX ? kMaxBasis : 1];
+    __shared__ int s_e;
     for (int i = threadIdx.x; i < k; i += blockDim.x) {
         double cx = 0, cy = 0;
         if (M) {
@@ -434,18 +534,24 @@ __global__ void __launch_bounds__(kRedThreads) basis_axpy_kernel(const VT* __res
         c.y = (A)cy;
         cs[i] = c;
         csn[i] = -c.y;
-        c3[0][i] = cy;
-        c3[1][i] = cx - cy;
-        c3[2][i] = cx + cy;
+        if (!FIX) {
+            c3[0][i] = cy;
+            c3[1][i] = cx - cy;
+            c3[2][i] = cx + cy;
+        }
     }
     __syncthreads();
+    int ec = 0;
+    if constexpr (FIX) ec = fix_coefs(cs, k, fc, &s_e);
     double nacc = 0;
     const long stride = (long)gridDim.x * blockDim.x;
     const long nn = off ? 0 : n;
     for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < nn; idx += stride) {
         A x0 = 0, y0 = 0;
         if (base) { const double2 bv = base[idx]; x0 = (A)bv.x; y0 = (A)bv.y; }
-        if (VM) {   // three-multiplication form: c a = (K1 + K2) + i (K1 + K3)
+        if constexpr (FIX) {
+            fix_update(V, ldv, k, idx, fc, ec, x0, y0);
+        } else if (VM) {   // three-multiplication form: c a = (K1 + K2) + i (K1 + K3)
             double k1 = 0, k2 = 0, k3 = 0;
 #pragma unroll 4
             for (int i = 0; i < k; i++) {
@@ -497,8 +603,8 @@ __global__ void __launch_bounds__(kRedThreads) basis_axpy_kernel(const VT* __res
 // pass).  Reduction vector 0 is ||w||^2, vectors 1 .. r the projections.  The last
 // block writes ||w||^2 to nrm2 and, when no second pass follows, 1 / ||w|| to dec.inv
 // and cf = M32 (V32^* w / ||w||) to dp.cf.
-template <int NGD>
-__global__ void __launch_bounds__(kRedThreads) cgs_update_defl_kernel(const double2* __restrict__ V, long ldv, int k,
+template <int NGD, bool FIX>
+__global__ void __launch_bounds__(kRedThreads, FIX ? 2 : 1) cgs_update_defl_kernel(const double2* __restrict__ V, long ldv, int k,
                                                                       const double2* __restrict__ coef,
                                                                       const double2* base, double2* out, long n,
                                                                       double2* nrm2, Dgks dec, int has_dec,
@@ -509,16 +615,22 @@ __global__ void __launch_bounds__(kRedThreads) cgs_update_defl_kernel(const doub
     if (off && !live) return;
     __shared__ double2 cs[kMaxBasis];
     __shared__ double csn[kMaxBasis];
-    __shared__ double c3[3][kMaxBasis];     // VM != NULL: Im c, Re c - Im c, Re c + Im c
+    __shared__ double c3[3][FIX ? 1 : kMaxBasis];     // VM != NULL: Im c, Re c - Im c, Re c + Im c
+    __shared__ FixCoef fc[FIX ? kMaxBasis : 1];
+    __shared__ int s_e;
     for (int i = threadIdx.x; i < k; i += blockDim.x) {
         const double2 c = make_double2(-coef[i].x, -coef[i].y);
         cs[i] = c;
         csn[i] = -c.y;
-        c3[0][i] = c.y;
-        c3[1][i] = c.x - c.y;
-        c3[2][i] = c.x + c.y;
+        if (!FIX) {
+            c3[0][i] = c.y;
+            c3[1][i] = c.x - c.y;
+            c3[2][i] = c.x + c.y;
+        }
     }
     __syncthreads();
+    int ec = 0;
+    if constexpr (FIX) ec = fix_coefs(cs, k, fc, &s_e);
     double nacc = 0;
     float dacc[NGD][16];
 #pragma unroll
@@ -530,7 +642,9 @@ __global__ void __launch_bounds__(kRedThreads) cgs_update_defl_kernel(const doub
     for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < nn; idx += stride) {
         double x0 = 0, y0 = 0;
         if (base) { const double2 bv = base[idx]; x0 = bv.x; y0 = bv.y; }
-        if (VM) {   // three-multiplication form: c a = (K1 + K2) + i (K1 + K3)
+        if constexpr (FIX) {
+            fix_update(V, ldv, k, idx, fc, ec, x0, y0);
+        } else if (VM) {   // three-multiplication form: c a = (K1 + K2) + i (K1 + K3)
             double k1 = 0, k2 = 0, k3 = 0;
 #pragma unroll 4
             for (int i = 0; i < k; i++) {
@@ -768,6 +882,9 @@ static RedShape red_shape(long n) {
     const long blocks = (n + threads - 1) / threads;
     return {(int)(blocks < 1 ? 1 : blocks), threads};
 }
+// Updates in fixed point: vectors of at least two rows per thread of a full launch (shorter
+// ones are bound by latency, which the conversions add to).
+static bool fix_rows(long n) { return n > 2l * red_blocks() * kRedThreads; }
 // Rows of the grid that share the groups of gv among nvt vectors: one, unless short vectors
 // leave SMs with fewer than 32 warps; then groups run side by side instead of one after
 // another.
@@ -817,11 +934,13 @@ die_status k_basis_axpy(const double2* V, long ldv, int k, const double2* coef, 
     const int has_dec = dec && dec->reorth ? 1 : 0;
     if (nrm2) {
         const RedShape sh = red_shape(n);
-        DIE_PROF(PK_UPDATE_NORM, st, launch_pdl(basis_axpy_kernel<double2, true>, dim3(sh.blocks), dim3(sh.threads), 0, st,
+        const auto kern = VM && fix_rows(n) ? basis_axpy_kernel<double2, true, true> : basis_axpy_kernel<double2, true, false>;
+        DIE_PROF(PK_UPDATE_NORM, st, launch_pdl(kern, dim3(sh.blocks), dim3(sh.threads), 0, st,
                      V, ldv, k, coef, sign, (const double2*)nullptr, (const double2*)nullptr, base, out, n, nrm2, d, has_dec, rs, skip, live ? 1 : 0, VM));
     } else {
         const int t = axpy_threads(n);
-        DIE_PROF(PK_LINCOMB, st, launch_pdl(basis_axpy_kernel<double2, false>, dim3(grid_for(n, t)), dim3(t), 0, st,
+        const auto kern = VM && fix_rows(n) ? basis_axpy_kernel<double2, false, true> : basis_axpy_kernel<double2, false, false>;
+        DIE_PROF(PK_LINCOMB, st, launch_pdl(kern, dim3(grid_for(n, t)), dim3(t), 0, st,
                      V, ldv, k, coef, sign, (const double2*)nullptr, (const double2*)nullptr, base, out, n, (double2*)nullptr, d, 0, rs, skip, 0, VM));
     }
     DIE_LAUNCH_CHECK();
@@ -831,7 +950,7 @@ die_status k_defl_update(const double2* V, long ldv, int r, const double2* M, co
                          double2* z, long n, const int* skip, cudaStream_t st) {
     if (r > kMaxBasis || r < 1) return DIE_EINVAL;
     const int t = axpy_threads(n);
-    DIE_PROF(PK_DEFL_UPDATE, st, launch_pdl(basis_axpy_kernel<double2, false>, dim3(grid_for(n, t)), dim3(t), 0, st,
+    DIE_PROF(PK_DEFL_UPDATE, st, launch_pdl(basis_axpy_kernel<double2, false, false>, dim3(grid_for(n, t)), dim3(t), 0, st,
                  V, ldv, r, (const double2*)nullptr, 1.0, M, s, x, z, n, (double2*)nullptr, Dgks{}, 0, RedScratch{}, skip, 0, (const double*)nullptr));
     DIE_LAUNCH_CHECK();
     return DIE_OK;
@@ -851,7 +970,8 @@ static die_status k_update_defl(const double2* V, long ldv, int k, const double2
     if (k > kMaxBasis || k < 0 || dp.r < 1 || dp.r > kDeflFoldMax) return DIE_EINVAL;
     const int ng = (dp.r + 7) / 8;
     const RedShape sh = red_shape(n);
-#define UPD_CASE(NG) DIE_PROF(PK_UPDATE_NORM, st, launch_pdl(cgs_update_defl_kernel<NG>, dim3(sh.blocks), dim3(sh.threads), 0, st, \
+    const bool fix = VM && fix_rows(n);
+#define UPD_CASE(NG) DIE_PROF(PK_UPDATE_NORM, st, launch_pdl(fix ? cgs_update_defl_kernel<NG, true> : cgs_update_defl_kernel<NG, false>, dim3(sh.blocks), dim3(sh.threads), 0, st, \
                               V, ldv, k, coef, (const double2*)w, w, n, nrm2, dec, has_dec, dp, rs, skip, live ? 1 : 0, VM))
     switch (ng) {
         case 1: UPD_CASE(1); break;
