@@ -838,7 +838,7 @@ def fp64_same_budget(op, b, step_iters, step_s, torch):
 
 
 def te_mag_rates(die, W, torch):
-    """The TE system with magnetic contrast (E1, E2, H3; three planes, runtime-plan kernels):
+    """The TE system with magnetic contrast (E1, E2, H3; three planes, any-grid kernels):
     regularised products per second at 512^2 (FP64 and complex64, back to back), and time to
     1e-6 on a magneto-dielectric core-shell at 128^2 (eps 4 + 0.2i core, 9 + 0.3i shell,
     mu_r = 2 + 0.1i in both, side 2 wavelengths): plain FP64 GMRES(40) against A_R A P^-1

@@ -78,8 +78,8 @@ typedef enum die_precision {
  * (the [A33]_nn of Section 4).  (The discrete relations A31 = -A13, A23 = -A32 printed in
  * Section 4 disagree with K31, K32 and are not used.)  The regulariser is A(chi'_e, chi_m),
  * chi'_e = 1/eps_r - 1: the symbol I + chi_e Q of Section 3 does not involve chi_m.  Its
- * products run on the runtime-plan kernels (no compile-time FFT path, no tile schedule, no
- * complex64 deflated first pass), and the learned preconditioner does not take it. */
+ * products have no tile schedule and no complex64 deflated first pass, and the learned
+ * preconditioner does not take it. */
 typedef enum die_polarization {
     DIE_TE = 0,
     DIE_TM = 1,

@@ -10,7 +10,8 @@
 // group order, so results do not depend on scheduling.  Updates: one thread per row,
 // sum over the basis with fused multiply-adds (4 per complex term); the optional norm
 // uses the same two-level reduction.  Every complex multiply-add is written as four
-// FMAs: on GB300 the FP64 pipe (about 2 FMA per clock per SM) bounds the FP64 kernels.
+// FMAs: on GB300 the FP64 pipe (about 2 FMA per clock per SM) bounds the FP64 kernels; updates
+// of long vectors run in fixed point instead (fix_update).
 #include "krylov.cuh"
 #include "prof.cuh"
 
