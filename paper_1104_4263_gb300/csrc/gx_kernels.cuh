@@ -201,14 +201,15 @@ __global__ void __launch_bounds__(P * (LS / gx_plan(LS).ept)) k2_gx(OpDev<float>
         const int k2 = t + fx_slot<EPT, p.r0>(e) * G;
         const bool neg2 = k2 > LS / 2;
         const int k2q = neg2 ? LS - k2 : k2;
-        float2 acc = make_float2(0.f, 0.f);
+        float2 acc;
 #pragma unroll
         for (int q = 0; q < P; q++) {
             const int pl = q == comp ? (q == 2 ? 5 : q) : (q + comp == 1 ? 2 : q + comp + 1);
             const bool neg = q != comp && (q + comp == 1 ? neg1 != neg2 : (q + comp == 2 ? neg2 : neg1));
             float2 w = __ldg(&g[pl * plane + k2q]);
             if (neg) w = make_float2(-w.x, -w.y);
-            acc = cadd(acc, cmul(w, bufs[q * Lp + pidx(k2)]));
+            const float2 z = cmul(w, bufs[q * Lp + pidx(k2)]);
+            acc = q == 0 ? z : cadd(acc, z);
         }
         x[e] = make_float2(acc.y, acc.x);
     }

@@ -37,7 +37,10 @@ namespace die {
 // Rows per block of the row passes: enough for 32-byte segments in the transposed
 // accesses (4 complex64), at most 512 threads per block.
 template <typename C> constexpr int tile_rows() { return sizeof(C) == 8 ? 4 : 2; }
-constexpr size_t kStageGreenMaxSmem = 200 * 1024;
+// The column pass stages its Green spectra where that leaves room for two blocks per SM
+// (not at length 4096: 119 KB with them, 70 KB without; two blocks of 128 registers there:
+// product at 2048^2 770 -> 704 us).
+constexpr size_t kStageGreenMaxSmem = 100 * 1024;
 
 template <typename C> __device__ __forceinline__ C czero() { C z; z.x = 0; z.y = 0; return z; }
 
@@ -229,7 +232,7 @@ __global__ void __launch_bounds__(512) k1_defl_fast(OpDev<float> op, DeflIn d, c
 // so the 2 x 2 Green multiply is done in registers between the two, with no shared-
 // memory round trip, and every twiddle serves both components.
 template <typename T, int L, bool RAG>
-__global__ void __launch_bounds__(L / 16, (L == 1024 ? 7 : 1)) k2_fast2(OpDev<T> op, C_t<T>* __restrict__ W,
+__global__ void __launch_bounds__(L / 16, (L == 1024 ? 7 : L == 4096 ? 2 : 1)) k2_fast2(OpDev<T> op, C_t<T>* __restrict__ W,
                                                                         int stage_g, const int* __restrict__ skip) {
     using C = C_t<T>;
     constexpr int G = L / 16, Q2 = L / 2 + 1, Lp = L + (L >> 4);
