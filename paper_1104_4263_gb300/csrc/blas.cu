@@ -10,8 +10,8 @@
 // group order, so results do not depend on scheduling.  Updates: one thread per row,
 // sum over the basis with fused multiply-adds (4 per complex term); the optional norm
 // uses the same two-level reduction.  Every complex multiply-add is written as four
-// FMAs: on GB300 the FP64 pipe (about 2 FMA per clock per SM) bounds the FP64 kernels; updates
-// of long vectors run in fixed point instead (fix_update).
+// FMAs: on GB300 the FP64 pipe (about 2 FMA per clock per SM) bounds the FP64 kernels; the
+// sweeps over long vectors run in fixed point instead (proj_fix_kernel, fix_update).
 #include "krylov.cuh"
 #include "prof.cuh"
 
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(kRedThreads, 2) proj3_kernel(const double2* __
     reduce_partials(rs, nvt, out, kGroup3);
 }
 
-// ---------------------------------------------------- fixed-point Gram-Schmidt updates
+// ----------------------------------------------------- fixed-point Gram-Schmidt sweeps
 // The update w - V h is a sum of products of FP64 numbers; GB300's FP64 pipe does 2 FMAs per
 // clock and SM, its integer pipes 24 32 x 32 -> 64-bit multiply-adds.  So a row's eight basis
 // values (of a common exponent) and their coefficients are brought to 58-bit integers, the
@@ -292,9 +292,8 @@ __global__ void __launch_bounds__(kRedThreads, 2) proj3_kernel(const double2* __
 // eight terms go through the FP64 pipe (4 operations instead of 24).  A term's error is 2^-58
 // of the largest term of its sum, below the 2^-53 of every term in FP64.  Complex products take
 // Gauss's three multiplications.  At 512^2 (cylinder, r = 8, 15 vectors on average) the update
-// takes 62 us where the FP64 form takes 92, bound by the conversions.  The projections gain
-// nothing from it (80 against 75 us: a chunk of rows needs its exponent before its first
-// product, and the loads wait on that) and stay in FP64.
+// takes 62 us where the FP64 form takes 92, bound by the conversions; the projections
+// (proj_fix_kernel), where a thread's rows share the exponent, 64 us for 75.
 constexpr int kGsBits = 58;                  // |operand| < 2^58, sums and differences < 2^59
 
 struct Fix { int h, l; };                    // h 2^32 + l, l signed
@@ -332,6 +331,94 @@ __device__ __forceinline__ double fix_add(double acc, const FixSum& s, int ea, i
     if (ea == 2047 || eb == 2047) return __longlong_as_double(0x7ff8000000000000ll);     // not finite
     if (e < -1022 || e > 960) return fix_add_far(acc, v, e);
     return fma(v, __hiloint2double((1023 + e) << 20, 0), acc);
+}
+
+// FP64 projections of long vectors in fixed point: conj(a) b = (P1 - P2) + i (P2 - P3),
+// P1 = a.x (b.x + b.y), P2 = (a.x - a.y) b.y, P3 = a.y (b.x - b.y), over chunks of R rows per
+// thread; a thread's R values of a vector share an exponent, and their sums (exact but for the
+// cut of fix_add) go to the thread's FP64 accumulators in shared memory, eight vectors to a
+// group.  The loop over the vectors is not unrolled: eight copies of its body do not fit the
+// instruction cache (80 us against 75 of the FP64 form at 512^2).  The norm stays in FP64.
+template <int R>
+__global__ void __launch_bounds__(kRedThreads, 2) proj_fix_kernel(const double2* __restrict__ V, long ldv, int nv,
+                                                                  const double2* __restrict__ w, long n,
+                                                                  int with_norm, double2* out, RedScratch rs,
+                                                                  const int* skip, int live) {
+    constexpr int K = 2 * kGroup3;
+    __shared__ double red[(kRedThreads / 32) * K];
+    __shared__ double2 sums[kGroup3][kRedThreads];
+    pdl_wait();
+    const bool off = block_flag(skip);
+    if (off && !live) return;
+    const int nvt = nv + (with_norm ? 1 : 0);
+    const long chunk = (long)kRedThreads * R, step = (long)gridDim.x * chunk;
+    for (int g0 = 0; g0 < nvt; g0 += kGroup3) {
+        if (off) { zero_partials(g0, K, nvt, rs); continue; }
+        const int nb = min(kGroup3, nv - g0);           // basis vectors of the group
+        const bool norm = g0 + kGroup3 > nv && nvt > nv;
+#pragma unroll
+        for (int v = 0; v < kGroup3; v++) sums[v][threadIdx.x] = make_double2(0.0, 0.0);
+        double nacc = 0;
+        for (long base = blockIdx.x * chunk + threadIdx.x; base < n + threadIdx.x; base += step) {
+            Fix by[R], bs[R], bd[R];
+            int ew = 0;
+            {
+                double2 b[R];
+#pragma unroll
+                for (int r = 0; r < R; r++) {
+                    const long idx = base + r * kRedThreads;
+                    b[r] = idx < n ? w[idx] : make_double2(0.0, 0.0);
+                }
+#pragma unroll
+                for (int r = 0; r < R; r++) {
+                    ew = max(ew, max(exp_field(b[r].x), exp_field(b[r].y)));
+                    if (norm) {
+                        nacc = fma(b[r].x, b[r].x, nacc);
+                        nacc = fma(b[r].y, b[r].y, nacc);
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < R; r++) {
+                    const long long x = fix_of(b[r].x, ew), y = fix_of(b[r].y, ew);
+                    by[r] = fix_split(y);
+                    bs[r] = fix_split(x + y);
+                    bd[r] = fix_split(x - y);
+                }
+            }
+#pragma unroll 1
+            for (int v = 0; v < nb; v++) {
+                const double2* src = V + (long)(g0 + v) * ldv + base;
+                double2 a[R];
+                int e = 0;
+#pragma unroll
+                for (int r = 0; r < R; r++)
+                    a[r] = base + r * kRedThreads < n ? src[r * kRedThreads] : make_double2(0.0, 0.0);
+#pragma unroll
+                for (int r = 0; r < R; r++) e = max(e, max(exp_field(a[r].x), exp_field(a[r].y)));
+                FixSum p1{0, 0}, p2{0, 0}, p3{0, 0};
+#pragma unroll
+                for (int r = 0; r < R; r++) {
+                    const long long x = fix_of(a[r].x, e), y = fix_of(a[r].y, e);
+                    fix_mac(p1, fix_split(x), bs[r]);
+                    fix_mac(p2, fix_split(x - y), by[r]);
+                    fix_mac(p3, fix_split(y), bd[r]);
+                }
+                double2 s = sums[v][threadIdx.x];
+                s.x = fix_add(s.x, FixSum{p1.hh - p2.hh, p1.mid - p2.mid}, e, ew);
+                s.y = fix_add(s.y, FixSum{p2.hh - p3.hh, p2.mid - p3.mid}, e, ew);
+                sums[v][threadIdx.x] = s;
+            }
+        }
+        double acc[K];
+#pragma unroll
+        for (int v = 0; v < kGroup3; v++) {
+            const double2 s = sums[v][threadIdx.x];
+            acc[2 * v] = norm && v == nv - g0 ? nacc : s.x;
+            acc[2 * v + 1] = s.y;
+        }
+        block_partials<double, K, kGroup3>(acc, red, g0, rs);
+    }
+    reduce_partials(rs, nvt, out);
 }
 
 // Runtime count -> compile-time CNT in [1, C].
@@ -883,9 +970,16 @@ static RedShape red_shape(long n) {
     const long blocks = (n + threads - 1) / threads;
     return {(int)(blocks < 1 ? 1 : blocks), threads};
 }
-// Updates in fixed point: vectors of at least two rows per thread of a full launch (shorter
+// Sweeps in fixed point: vectors of at least two rows per thread of a full launch (shorter
 // ones are bound by latency, which the conversions add to).
 static bool fix_rows(long n) { return n > 2l * red_blocks() * kRedThreads; }
+// Rows per thread and chunk of the fixed-point projections: four while one chunk per block
+// holds the vector, seven beyond (one chunk per block at 512^2, 96% of the threads used there).
+static int proj_rows(long n) { return n <= 4l * red_blocks() * kRedThreads ? 4 : 7; }
+static int proj_blocks(long n) {
+    const long chunk = (long)proj_rows(n) * kRedThreads, b = (n + chunk - 1) / chunk;
+    return (int)(b < red_blocks() ? b : red_blocks());
+}
 // Rows of the grid that share the groups of gv among nvt vectors: one, unless short vectors
 // leave SMs with fewer than 32 warps; then groups run side by side instead of one after
 // another.
@@ -912,7 +1006,9 @@ die_status k_dots(const double2* V, long ldv, int nv, const double2* w, long n, 
     if (nv + 1 > kMaxBasis || nv < 0) return DIE_EINVAL;
     const RedShape sh = red_shape(n);
     const int nvt = nv + (with_norm ? 1 : 0);
-    if (VM)
+    if (VM && fix_rows(n))
+        DIE_PROF(PK_DOTS, st, launch_pdl(proj_rows(n) == 4 ? proj_fix_kernel<4> : proj_fix_kernel<7>, dim3(proj_blocks(n)), dim3(kRedThreads), 0, st, V, ldv, nv, w, n, with_norm, out, rs, skip, live ? 1 : 0));
+    else if (VM)
         DIE_PROF(PK_DOTS, st, launch_pdl(proj3_kernel, dim3(sh.blocks, red_rows(sh, nvt, kGroup3)), dim3(sh.threads), 0, st, V, VM, ldv, nv, w, n, with_norm, out, rs, skip, live ? 1 : 0));
     else
         DIE_PROF(PK_DOTS, st, launch_pdl(proj_kernel<double2, kGroupFp64>, dim3(sh.blocks, red_rows(sh, nvt, kGroupFp64)), dim3(sh.threads), 0, st, V, ldv, nv, w, n, with_norm, out, rs, skip, live ? 1 : 0));

@@ -8,8 +8,8 @@
 // single-pass (the second-pass kernels are not launched); a
 // cycle in which the criterion fires stops and runs again with the second passes, and
 // the solve keeps them.  The passes use the three-multiplication form of the complex
-// products (Re - Im of every basis vector is stored when the vector is normalised; the updates
-// of long vectors form it in fixed point).
+// products (Re - Im of every basis vector is stored when the vector is normalised; the sweeps
+// over long vectors work in fixed point and do without it).
 // The new Hessenberg column is rotated by Givens rotations on the device, on a side
 // stream one step behind, since the next Arnoldi step does not need the rotations; the
 // normalisation of the new vector uses 1 / ||w|| from the last Gram-Schmidt kernel.
