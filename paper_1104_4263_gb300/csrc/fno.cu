@@ -46,6 +46,8 @@ struct fno_s {
     float* part = nullptr;          // partial sums of weight and bias gradients
     long part_cap = 0;
     bool expanded = false;          // Rr holds the current parameters
+    bool captured = false;          // a training step was captured: replays change the parameters
+                                    // unseen, so Rr is formed on every pass from then on
     cudaStream_t side = nullptr;    // weight gradients of the backward pass
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int spare = 0;                  // CTA slots the backward pass leaves to the side stream
@@ -420,7 +422,7 @@ die_status layer_backward(fno_s* f, int l, int B, const float* hin, const float*
 
 // Rr from the parameters, once per change of them.
 die_status expand_weights(fno_s* f, cudaStream_t st) {
-    if (f->expanded) return DIE_OK;
+    if (f->expanded && !f->captured) return DIE_OK;
     const long per = (long)f->NM * 4 * f->C * f->C;
     for (int l = 0; l < f->L; l++)
         DIE_TRY(run(expand_r_kernel, dim3(f->C, (f->m * f->m + kModeTile - 1) / kModeTile, 2), kT,
@@ -729,6 +731,9 @@ extern "C" die_status fno_train_step(fno_t f, int B, const float* x, const float
                                      void* stream) {
     if (!f || !x || !t || B < 1 || B > f->maxB || !(lr >= 0)) return DIE_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    DIE_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+    if (cap != cudaStreamCaptureStatusNone) f->captured = true;
     const long n = (long)B * f->cout * f->HW;
     DIE_TRY(forward(f, B, x, f->ytmp, st));
     // gradient in place of y
