@@ -53,18 +53,17 @@ WORKLOAD = ("core-shell 512x512 (eps -2+0.1i core R1.5, 20+0.5i shell R2.5, side
             "FP32 products + FP64 Krylov, 1500 Arnoldi steps per step")
 L2_NOTE = "working set > L2 (Krylov basis 31 x 8.4 MB, deflation basis 20 x 4.2 MB)"
 # ncu DRAM bytes (read + write) of one launch of the FP64 projection kernel on this
-# workload: 13 basis vectors with their Re - Im planes, and the norm of w, over
-# 2N = 524288, from one capture of the committed profile driver (bench.py
-# --profile-driver; the kernel is unchanged since).  Its traffic grows with the vectors
+# workload: 13 basis vectors (16 B a value) and the norm of w, over 2N = 524288, from one
+# capture of the committed profile driver (bench.py --profile-driver).  Its traffic grows with the vectors
 # read, so it is scaled to the bench's average launch by the algorithmic bytes.
 # DRAM bytes of the five passes of one complex64 regularised product at 512^2 (reads; no
 # DRAM writes were counted during the passes: the row spectra stay in L2)
 NCU_PRODUCT = {"dram_bytes": (6.315520 + 14.774016 + 14.725632 + 14.769408 + 12.608512) * 1e6, "n": 524288,
                "source": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum -k regex:\"k1_fast|k2_fast2|"
                          "k3k1_fast|k3_fast\" -c 5 on bench.py --profile-driver (its first complex64 product)"}
-NCU_DOTS = {"dram_bytes": 175.365632e6 + 0.137216e6, "nv": 13, "n": 524288,
-            "source": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum -k regex:proj3 -s 10 -c 3 on "
-                      "bench.py --profile-driver (the 13-vector launch; groups of eight vectors)"}
+NCU_DOTS = {"dram_bytes": 118.963456e6 + 3.052032e6, "nv": 13, "n": 524288,
+            "source": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum -k regex:proj_fix on "
+                      "bench.py --profile-driver (the 13-vector launch; groups of seven vectors)"}
 
 
 def fp64_peak(die):
@@ -269,9 +268,10 @@ def work_model(cls, p, op, r, steps_per_cycle, cycles, products, fp64_products):
         return "hbm", cycles * (r * n * 16 + 2 * n * 16)
     m = steps_per_cycle
     if cls == "dots_bytes":
-        # step j: j+1 basis vectors (16 B) and their Re - Im planes (8 B), w read once;
-        # per cycle the residual norm and the FP64 deflation projections (r vectors + x)
-        per_cycle = sum((j + 1) * 24 + 16 for j in range(m)) + 16 + 16 * r + 16
+        # step j: j+1 basis vectors (16 B; the fixed-point sweeps of long vectors do not read
+        # their Re - Im planes), w read once; per cycle the residual norm and the FP64
+        # deflation projections (r vectors + x)
+        per_cycle = sum((j + 1) * 16 + 16 for j in range(m)) + 16 + 16 * r + 16
         return "hbm", cycles * per_cycle * n + 16 * n
     if cls == "dots":
         # step j of a cycle: j+1 projections + the norm of w; per cycle one norm of the
@@ -503,7 +503,7 @@ def main():
             if best == "dots" and NCU_DOTS and 2 * p.N == NCU_DOTS["n"]:
                 _, tot_bytes = work_model("dots_bytes", p, op, D.r, RESTART, cycles, prof_products, fp64_products)
                 alg_bytes = tot_bytes / k["launches"]
-                captured_alg = (NCU_DOTS["nv"] * 24 + 16) * NCU_DOTS["n"]
+                captured_alg = (NCU_DOTS["nv"] * 16 + 16) * NCU_DOTS["n"]
                 out["roofline"]["traffic"] = NCU_DOTS["dram_bytes"] * alg_bytes / captured_alg
                 out["roofline"]["algorithmic_bytes_per_launch"] = alg_bytes
                 out["roofline"]["traffic_source"] = (NCU_DOTS["source"] + ", scaled to the average launch by the "
