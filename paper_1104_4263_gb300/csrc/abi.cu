@@ -61,6 +61,12 @@ bool make_plan(int L, FftPlan* p) {
     return true;
 }
 
+static FftPlan reversed(const FftPlan& f) {
+    FftPlan r = f;
+    for (int s = 0; s < f.ns; s++) r.radix[s] = f.radix[f.ns - 1 - s];
+    return r;
+}
+
 int choose_fft_size(int n) {
     int best = 0;
     for (int L = 16; L <= 4096; L *= 2) {
@@ -291,6 +297,8 @@ static die_status create_impl(const dieop_desc* desc, const void* eps_r, int eps
     if (op->M1 < 2 * op->n1 || op->M2 < 2 * op->n2) return DIE_EINVAL;
     if (!make_plan(op->M1, &op->f1) || !make_plan(op->M2, &op->f2)) return DIE_EUNSUPPORTED;
     if (op->M1 > 4096 || op->M2 > 4096) return DIE_EUNSUPPORTED;
+    op->i1 = reversed(op->f1);
+    op->i2 = reversed(op->f2);
     op->Q1 = op->M1 / 2 + 1;
     op->Q2 = op->M2 / 2 + 1;
     DIE_CUDA_TRY(cudaGetDevice(&op->device));

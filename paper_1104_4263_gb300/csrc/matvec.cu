@@ -21,10 +21,11 @@ static FxDev view_d(const dieop_s* op) {
 OpDev<float> view_f(const dieop_s* op) {
     OpDev<float> v{};
     v.n1 = op->n1; v.n2 = op->n2; v.M1 = op->M1; v.M2 = op->M2; v.Q1 = op->Q1; v.Q2 = op->Q2;
+    v.f1 = op->f1; v.i1 = op->i1; v.f2 = op->f2; v.i2 = op->i2;
     v.planes = op->planes;
     v.xs = (long)op->planes * op->n1 * op->n2;
     v.ws = (long)op->planes * op->M1 * op->n2;
-    v.gq = op->gq_f;
+    v.tw1 = op->tw1_f; v.tw2 = op->tw2_f; v.gq = op->gq_f;
     v.twx1 = op->tw1_f + op->M1; v.twx2 = op->tw2_f + op->M2;
     v.gx1 = op->tw1_f + 3 * (size_t)op->M1; v.gx2 = op->tw2_f + 3 * (size_t)op->M2;
     v.tr = op->tile_rows_c64;
