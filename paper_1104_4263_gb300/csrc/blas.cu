@@ -295,6 +295,9 @@ __global__ void __launch_bounds__(kRedThreads, 2) proj3_kernel(const double2* __
 // takes 62 us where the FP64 form takes 92, bound by the conversions; the projections
 // (proj_fix_kernel), where a thread's rows share the exponent, 64 us for 75.
 constexpr int kGsBits = 58;                  // |operand| < 2^58, sums and differences < 2^59
+// Least common exponent field of a group of operands: from 2^-958 of its bound down, a value
+// counts in units of 2^-1016, so that zeros (field 0, no leading bit) shift out whole.
+constexpr int kFixLeast = 64;
 
 struct Fix { int h, l; };                    // h 2^32 + l, l signed
 __device__ __forceinline__ Fix fix_split(long long a) {
@@ -304,8 +307,8 @@ __device__ __forceinline__ Fix fix_split(long long a) {
     return f;
 }
 __device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >> 20) & 2047; }
-// v 2^(1022 + kGsBits - emax) towards zero, for a v whose exponent field is at most emax (so |v| <
-// 2^(emax - 1022)).  Zeros and values below 2^-63 of the largest give 0.
+// v 2^(1022 + kGsBits - emax) towards zero, for a v whose exponent field is at most emax >=
+// kFixLeast (so |v| < 2^(emax - 1022)).  Zeros, subnormal numbers and values below one unit give 0.
 __device__ __forceinline__ long long fix_of(double v, int emax) {
     const int hi = __double2hiint(v);
     const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u, ml = (unsigned)__double2loint(v);
@@ -329,7 +332,7 @@ __device__ __forceinline__ double fix_add(double acc, const FixSum& s, int ea, i
     const double v = __ll2double_rn((s.hh << 5) + (s.mid >> 27));
     const int e = ea + eb - 2 * (1022 + kGsBits) + 59;
     if (ea == 2047 || eb == 2047) return __longlong_as_double(0x7ff8000000000000ll);     // not finite
-    if (e < -1022 || e > 960) return fix_add_far(acc, v, e);
+    if (e < -1022 || e > 960) return v == 0.0 ? acc : fix_add_far(acc, v, e);
     return fma(v, __hiloint2double((1023 + e) << 20, 0), acc);
 }
 
@@ -361,7 +364,7 @@ __global__ void __launch_bounds__(kRedThreads, 2) proj_fix_kernel(const double2*
         double nacc = 0;
         for (long base = blockIdx.x * chunk + threadIdx.x; base < n + threadIdx.x; base += step) {
             Fix by[R], bs[R], bd[R];
-            int ew = 0;
+            int ew = kFixLeast;
             {
                 double2 b[R];
 #pragma unroll
@@ -389,7 +392,7 @@ __global__ void __launch_bounds__(kRedThreads, 2) proj_fix_kernel(const double2*
             for (int v = 0; v < nb; v++) {
                 const double2* src = V + (long)(g0 + v) * ldv + base;
                 double2 a[R];
-                int e = 0;
+                int e = kFixLeast;
 #pragma unroll
                 for (int r = 0; r < R; r++)
                     a[r] = base + r * kRedThreads < n ? src[r * kRedThreads] : make_double2(0.0, 0.0);
@@ -541,7 +544,7 @@ __device__ __forceinline__ double inv_norm(double s2) {
 // in fixed point of one exponent.  All threads call it; k <= kMaxBasis.
 struct FixCoef { Fix f[3]; };
 __device__ __forceinline__ int fix_coefs(const double2* c, int k, FixCoef* fc, int* s_e) {
-    if (threadIdx.x == 0) *s_e = 0;
+    if (threadIdx.x == 0) *s_e = kFixLeast;
     __syncthreads();
     int e = 0;
     for (int i = threadIdx.x; i < k; i += blockDim.x) e = max(e, max(exp_field(c[i].x), exp_field(c[i].y)));
@@ -564,7 +567,7 @@ __device__ __forceinline__ void fix_update(const double2* __restrict__ V, long l
 #pragma unroll 1
     for (int i0 = 0; i0 < k; i0 += GV) {
         double2 a[GV];
-        int e = 0;
+        int e = kFixLeast;
 #pragma unroll
         for (int v = 0; v < GV; v++) a[v] = i0 + v < k ? V[(long)(i0 + v) * ldv + idx] : make_double2(0.0, 0.0);
 #pragma unroll
