@@ -45,7 +45,8 @@ struct fno_s {
     float *g1 = nullptr, *g2 = nullptr, *g3 = nullptr;   // backward scratch B x max(C, hid) x HW
     float* part = nullptr;          // partial sums of weight and bias gradients
     long part_cap = 0;
-    bool expanded = false;          // Rr holds the current parameters
+    bool expanded = false;          // Rr holds the current parameters: set only by a pass that was
+                                    // launched (not recorded) on the parameters, cleared by any error
     bool captured = false;          // a training step was captured: replays change the parameters
                                     // unseen, so Rr is formed on every pass from then on
     cudaStream_t side = nullptr;    // weight gradients of the backward pass
@@ -420,19 +421,30 @@ die_status layer_backward(fno_s* f, int l, int B, const float* hin, const float*
     return tc_gemm(g, st);
 }
 
-// Rr from the parameters, once per change of them.
+die_status is_capturing(cudaStream_t st, bool* cap) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    DIE_CUDA_TRY(cudaStreamIsCapturing(st, &s));
+    *cap = s != cudaStreamCaptureStatusNone;
+    return DIE_OK;
+}
+
+// Rr from the parameters, once per change of them.  On a capturing stream the work is only
+// recorded: it is always part of the recording, and says nothing about Rr's contents.
 die_status expand_weights(fno_s* f, cudaStream_t st) {
-    if (f->expanded && !f->captured) return DIE_OK;
+    bool cap = false;
+    DIE_TRY(is_capturing(st, &cap));
+    if (f->expanded && !f->captured && !cap) return DIE_OK;
+    f->expanded = false;
     const long per = (long)f->NM * 4 * f->C * f->C;
     for (int l = 0; l < f->L; l++)
         DIE_TRY(run(expand_r_kernel, dim3(f->C, (f->m * f->m + kModeTile - 1) / kModeTile, 2), kT,
                     (size_t)f->C * (kModeTile + 1) * sizeof(float2), st, (const float*)f->params + f->oR1[l],
                     (const float*)f->params + f->oR2[l], f->Rr + (long)l * per, f->C, f->m, f->MH));
-    f->expanded = true;
+    f->expanded = !cap;
     return DIE_OK;
 }
 
-die_status forward(fno_s* f, int B, const float* x, float* y, cudaStream_t st) {
+die_status forward_passes(fno_s* f, int B, const float* x, float* y, cudaStream_t st) {
     const int C = f->C, HW = f->HW;
     const long CHW = (long)C * HW, HHW = (long)f->hid * HW;
     float* prm = f->params;
@@ -452,6 +464,12 @@ die_status forward(fno_s* f, int B, const float* x, float* y, cudaStream_t st) {
                  (long)f->cout * HW, prm + f->oq2, st));
     f->lastB = B;
     return DIE_OK;
+}
+
+die_status forward(fno_s* f, int B, const float* x, float* y, cudaStream_t st) {
+    const die_status s = forward_passes(f, B, x, y, st);
+    if (s != DIE_OK) f->expanded = false;
+    return s;
 }
 
 die_status backward_passes(fno_s* f, int B, const float* gy, float* gx, cudaStream_t st) {
@@ -612,12 +630,20 @@ die_status create_impl(const fno_desc* d, fno_s* f) {
     return make_dft(f);
 }
 
-// Reads (and clears) the flag a GEMM sets when one of its bounded waits gave up.
+// Reads (and clears) the flag a GEMM sets when one of its bounded waits gave up.  A capturing
+// stream refuses the synchronisation; that error is this call's, not one for the next call's
+// launch check.
 die_status check_err(fno_s* f, cudaStream_t st) {
     int e = 0;
-    DIE_CUDA_TRY(cudaMemcpyAsync(&e, f->err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    DIE_CUDA_TRY(cudaStreamSynchronize(st));
-    if (!e) return DIE_OK;
+    cudaError_t r = cudaMemcpyAsync(&e, f->err, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (r == cudaSuccess) r = cudaStreamSynchronize(st);
+    if (r == cudaSuccess && !e) return DIE_OK;
+    f->expanded = false;
+    if (r != cudaSuccess) {
+        cudaGetLastError();
+        set_last_cuda_error(r, "network pass", __FILE__, __LINE__);
+        return DIE_ECUDA;
+    }
     DIE_CUDA_TRY(cudaMemsetAsync(f->err, 0, sizeof(int), st));
     return DIE_ETIMEOUT;
 }
@@ -731,9 +757,9 @@ extern "C" die_status fno_train_step(fno_t f, int B, const float* x, const float
                                      void* stream) {
     if (!f || !x || !t || B < 1 || B > f->maxB || !(lr >= 0)) return DIE_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    DIE_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
-    if (cap != cudaStreamCaptureStatusNone) f->captured = true;
+    bool cap = false;
+    DIE_TRY(is_capturing(st, &cap));
+    if (cap) f->captured = true;
     const long n = (long)B * f->cout * f->HW;
     DIE_TRY(forward(f, B, x, f->ytmp, st));
     // gradient in place of y
