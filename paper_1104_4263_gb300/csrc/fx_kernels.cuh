@@ -21,8 +21,8 @@ namespace die {
 constexpr int kFxTileRows = 2;    // rows per block: 32-byte segments in the transposed accesses
 
 // Magnitudes of a transform's values z: mx >= max (|re| + |im|) and s >= sum (|re| + |im|),
-// both times 2^(1023 - e) (FP64 inputs; e is the largest exponent field) or over 2^38
-// (fixed-point values, e unused).
+// both times 2^(1023 - e) (FP64 inputs; e is the largest exponent field, 1 where the largest
+// number is subnormal, 0 where all are zeros) or over 2^38 (fixed-point values, e unused).
 struct FxNorm { int e; float mx, s; };
 
 __device__ __forceinline__ int fx_mag_hi(double v) { return __double2hiint(v) & 0x7fffffff; }
@@ -42,6 +42,13 @@ template <int EPT, typename K> __device__ __forceinline__ FxNorm fx_norm(const d
     for (int e = 0; e < EPT; e++)
         if (keep(e)) m = max(m, max(fx_mag_hi(v[e].x), fx_mag_hi(v[e].y)));
     FxNorm a{m >> 20, 0.f, 0.f};
+    if (a.e == 0) {
+        int any = m;
+#pragma unroll
+        for (int e = 0; e < EPT; e++)
+            if (keep(e)) any |= __double2loint(v[e].x) | __double2loint(v[e].y);
+        if (any) a.e = 1;
+    }
 #pragma unroll
     for (int e = 0; e < EPT; e++)
         if (keep(e)) {
@@ -107,7 +114,6 @@ __device__ __forceinline__ FxScale fx_scale(const FxNorm& a, int r0, int r1, int
     s.bad = a.e == 2047;
     s.slow = a.e != 0 && (a.e < 123 || a.e > 1923);
     const float b = (float)(a.e - 1023);
-    // no normal number among the values: taken as zeros
     s.lm = __log2f(a.mx) + b;
     s.ls = __log2f(a.s) + b;
     s.e = a.e == 0 ? 0 : fx_room(r0, r1, q, half, s.lm, s.ls, 0);
