@@ -404,8 +404,9 @@ __global__ void __launch_bounds__(512) k3k1_fx(FxDev op, double2* __restrict__ W
 
 // ------------------------------------------------------------------------- K2
 // One block per column k1, G threads per plane.  One scale for the planes of the column
-// (their products are added), raised to the largest value before the Green multiply and
-// chosen anew for each plane's inverse transform.
+// (their products are added; each its own where the planes are not coupled, so that none
+// loses bits to a larger one), raised to the largest value before the Green multiply and chosen
+// anew for each plane's inverse transform.
 // Blocks per SM that keep a thread's registers at 128 (16 warps), or at 80 with 8 values.
 constexpr int fx_k2_blocks(int threads, int ept) {
     return threads <= 512 ? (ept == 8 ? 24 : 16) / ((threads + 31) / 32) : 1;
@@ -432,14 +433,15 @@ __global__ void __launch_bounds__(MAXT, fx_k2_blocks(MAXT, EPT)) k2_fx(FxDev op,
     const long plane = (long)op.Q1 * Q2;
     const fxw* g = op.gx + (long)k1q * Q2;
     auto low = [](int e) { return fx_slot<EPT, R0>(e) < EPT / 2; };
-    // the planes' norms, merged over the planes (largest sum)
+    // the planes' norms, merged over the planes (largest sum); a value that is not finite makes
+    // every plane so
     auto over_planes = [&](FxNorm a, FxNorm* rp) {
         if (t == 0) rp[comp] = a;
         __syncthreads();
-        a = rp[0];
+        FxNorm r = rp[0];
 #pragma unroll
-        for (int p = 1; p < P; p++) a = fx_merge(a, rp[p], false);
-        return a;
+        for (int p = 1; p < P; p++) r = fx_merge(r, rp[p], false);
+        return P == 2 && op.apart && r.e != 2047 ? a : r;
     };
     fxc x[EPT];
     FxScale s;

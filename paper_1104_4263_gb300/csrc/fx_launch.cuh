@@ -16,6 +16,7 @@ struct FxDev {
     const double2* chim;          // magnetic contrast (three planes)
     long xs, ws;                  // batched products: elements per vector and per set of row spectra
     int planes;
+    bool apart;                   // no coupling between the planes (TM)
 };
 
 // First row pass of a product on a vector that is still to be normalised: v *= *inv in place

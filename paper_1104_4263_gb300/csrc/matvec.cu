@@ -14,6 +14,7 @@ static FxDev view_d(const dieop_s* op) {
     v.gx = op->gx; v.ge = op->ge;
     v.chim = op->chim_d;
     v.planes = op->planes;
+    v.apart = op->pol == DIE_TM;
     v.xs = (long)op->planes * op->n1 * op->n2;
     v.ws = (long)op->planes * op->M1 * op->n2;
     return v;
