@@ -591,8 +591,10 @@ __device__ __forceinline__ void fix_update(const double2* __restrict__ V, long l
 // out = base + sum_i V_i c_i.  Coefficients: c = sign * coef, or c = M s when M != NULL.
 // The sum for a row starts from base and runs through the basis in order in one pair of
 // accumulators (the FP64 pipe, not the FMA latency, bounds the loop).
+// FIX: the fixed-point form, at two blocks per SM (no bound otherwise: with one of 1 the compiler
+// takes 82 registers for 48, and the deflation update of 9 vectors at 512^2 45 us for 41).
 template <typename VT, bool NORM, bool FIX>
-__global__ void __launch_bounds__(kRedThreads, FIX ? 2 : 1) basis_axpy_kernel(const VT* __restrict__ V, long ldv, int k,
+__global__ void __launch_bounds__(kRedThreads, FIX ? 2 : 0) basis_axpy_kernel(const VT* __restrict__ V, long ldv, int k,
                                                                  const double2* __restrict__ coef, double sign,
                                                                  const double2* __restrict__ M,
                                                                  const double2* __restrict__ s, const double2* base,
@@ -695,7 +697,7 @@ __global__ void __launch_bounds__(kRedThreads, FIX ? 2 : 1) basis_axpy_kernel(co
 // block writes ||w||^2 to nrm2 and, when no second pass follows, 1 / ||w|| to dec.inv
 // and cf = M32 (V32^* w / ||w||) to dp.cf.
 template <int NGD, bool FIX>
-__global__ void __launch_bounds__(kRedThreads, FIX ? 2 : 1) cgs_update_defl_kernel(const double2* __restrict__ V, long ldv, int k,
+__global__ void __launch_bounds__(kRedThreads, FIX ? 2 : 0) cgs_update_defl_kernel(const double2* __restrict__ V, long ldv, int k,
                                                                       const double2* __restrict__ coef,
                                                                       const double2* base, double2* out, long n,
                                                                       double2* nrm2, Dgks dec, int has_dec,
