@@ -80,18 +80,19 @@ __device__ __forceinline__ void block_partials(A (&acc)[K], A* red, int g0, cons
 }
 
 // Final sums of the per-block partials partial[i * gridDim.x + b] (see RedScratch) of the
-// vectors this block's row of the grid works on: all i < nv, or, when gridDim.y > 1, the
-// groups y, y + gridDim.y, ... of gv vectors.  Every thread of every block calls it after its
-// block's partials are written; it returns true in the one block (of each grid row) that
-// has written their sums to out, whose threads may then read them.
-__device__ bool reduce_partials(const RedScratch& rs, int nv, double2* out, int gv = kMaxBasis) {
+// vectors this block's row of the grid works on: all i < nv, or (GV > 0) the groups y,
+// y + gridDim.y, ... of GV vectors.  Every thread of every block calls it after its block's
+// partials are written; it returns true in the one block (of each grid row) that has written
+// their sums to out, whose threads may then read them.
+template <int GV = 0> __device__ bool reduce_partials(const RedScratch& rs, int nv, double2* out) {
     __shared__ int s_last;
     const int G = gridDim.x, ng = (G + kRedGroup - 1) / kRedGroup, g = blockIdx.x / kRedGroup;
     const int gsz = min(kRedGroup, G - g * kRedGroup);
-    const int y = blockIdx.y, gy = gridDim.y;
+    const int y = GV ? blockIdx.y : 0, gy = GV ? gridDim.y : 1;
+    constexpr int gv = GV ? GV : 1;
     unsigned* counter = rs.counter + y * (1 + kRedGroupsMax);
-    const int nl = gy == 1 ? nv : ((nv + gv - 1) / gv - y + gy - 1) / gy * gv;   // local vector slots
-    auto vec = [&](int l) { return gy == 1 ? l : (l / gv * gy + y) * gv + l % gv; };
+    const int nl = GV ? ((nv + gv - 1) / gv - y + gy - 1) / gy * gv : nv;   // local vector slots
+    auto vec = [&](int l) { return GV ? (l / gv * gy + y) * gv + l % gv : l; };
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -106,7 +107,7 @@ __device__ bool reduce_partials(const RedScratch& rs, int nv, double2* out, int 
     double* p2 = reinterpret_cast<double*>(rs.partial2);
     for (int e = threadIdx.x; e < 2 * nl; e += blockDim.x) {   // e = 2 l + component
         const int i = vec(e >> 1);
-        if (i >= nv) continue;
+        if (GV && i >= nv) continue;
         const double* src = pp + 2 * ((long)i * G + (long)g * kRedGroup) + (e & 1);
         double s = 0;
         for (int b = 0; b < gsz; b++) s += __ldcg(src + 2 * b);
@@ -125,7 +126,7 @@ __device__ bool reduce_partials(const RedScratch& rs, int nv, double2* out, int 
     double* o = reinterpret_cast<double*>(out);
     for (int e = threadIdx.x; e < 2 * nl; e += blockDim.x) {
         const int i = vec(e >> 1);
-        if (i >= nv) continue;
+        if (GV && i >= nv) continue;
         const double* src = p2 + 2 * (long)i * ng + (e & 1);
         double s = 0;
         for (int q = 0; q < ng; q++) s += __ldcg(src + 2 * q);
@@ -263,8 +264,10 @@ __device__ __forceinline__ void proj_group3_n(int cnt, const double2* V, const d
     else if constexpr (C > 1) proj_group3_n<C - 1>(cnt, V, VM, ldv, g0, nv, w, n, red, rs);
 }
 
-// FP64 projections in the three-multiplication form, kGroup3 vectors per pass.
+// FP64 projections in the three-multiplication form, kGroup3 vectors per pass.  ROWS: the
+// groups are shared by the rows of the grid (red_rows).
 constexpr int kGroup3 = 8;
+template <bool ROWS>
 __global__ void __launch_bounds__(kRedThreads, 2) proj3_kernel(const double2* __restrict__ V,
                                                                const double* __restrict__ VM, long ldv, int nv,
                                                                const double2* __restrict__ w, long n, int with_norm,
@@ -276,12 +279,12 @@ __global__ void __launch_bounds__(kRedThreads, 2) proj3_kernel(const double2* __
     const bool off = block_flag(skip);
     if (off && !live) return;
     const int nvt = nv + (with_norm ? 1 : 0);
-    for (int g0 = blockIdx.y * kGroup3; g0 < nvt; g0 += gridDim.y * kGroup3) {
+    for (int g0 = ROWS ? blockIdx.y * kGroup3 : 0; g0 < nvt; g0 += (ROWS ? gridDim.y : 1) * kGroup3) {
         if (off) { zero_partials(g0, 2 * kGroup3, nvt, rs); continue; }
         const int cnt = nvt - g0 < kGroup3 ? nvt - g0 : kGroup3;
         proj_group3_n<kGroup3>(cnt, V, VM, ldv, g0, nv, w, n, red, rs);
     }
-    reduce_partials(rs, nvt, out, kGroup3);
+    reduce_partials<ROWS ? kGroup3 : 0>(rs, nvt, out);
 }
 
 // ----------------------------------------------------- fixed-point Gram-Schmidt sweeps
@@ -435,7 +438,7 @@ __device__ __forceinline__ void proj_group_n(int cnt, const VT* V, long ldv, int
 
 // out[i] = sum_e conj(V_i[e]) w[e] for i < nv; with_norm: out[nv] = ||w||^2 (as the
 // projection of w on itself).  Groups of GV vectors; w is re-read once per group.
-template <typename VT, int GV>
+template <typename VT, int GV, bool ROWS>
 __global__ void __launch_bounds__(kRedThreads) proj_kernel(const VT* __restrict__ V, long ldv, int nv,
                                                            const VT* __restrict__ w, long n, int with_norm,
                                                            double2* out, RedScratch rs, const int* skip, int live) {
@@ -446,12 +449,12 @@ __global__ void __launch_bounds__(kRedThreads) proj_kernel(const VT* __restrict_
     const bool off = block_flag(skip);
     if (off && !live) return;
     const int nvt = nv + (with_norm ? 1 : 0);
-    for (int g0 = blockIdx.y * GV; g0 < nvt; g0 += gridDim.y * GV) {
+    for (int g0 = ROWS ? blockIdx.y * GV : 0; g0 < nvt; g0 += (ROWS ? gridDim.y : 1) * GV) {
         if (off) { zero_partials(g0, K, nvt, rs); continue; }
         const int cnt = nvt - g0 < GV ? nvt - g0 : GV;
         proj_group_n<VT, GV, false>(cnt, V, ldv, g0, nv, w, nullptr, nullptr, 1.0, n, red, rs);
     }
-    reduce_partials(rs, nvt, out, GV);
+    reduce_partials<ROWS ? GV : 0>(rs, nvt, out);
 }
 
 // Deflation projections of the FP32-inner solves (see k_dots32): complex64 basis and
@@ -978,18 +981,37 @@ static RedShape red_shape(long n) {
 // Sweeps in fixed point: vectors of at least two rows per thread of a full launch (shorter
 // ones are bound by latency, which the conversions add to).
 static bool fix_rows(long n) { return n > 2l * red_blocks() * kRedThreads; }
-// Rows per thread and chunk of the fixed-point projections: four while one chunk per block
-// holds the vector, seven beyond (one chunk per block at 512^2, 96% of the threads used there).
-static int proj_rows(long n) { return n <= 4l * red_blocks() * kRedThreads ? 4 : 7; }
-static int proj_blocks(long n) {
-    const long chunk = (long)proj_rows(n) * kRedThreads, b = (n + chunk - 1) / chunk;
-    return (int)(b < red_blocks() ? b : red_blocks());
+// Rows per thread and chunk, and blocks, of the fixed-point projections: the rows that leave the
+// busiest SM the least to do.  A chunk costs its rows and about one more (its exponent, the sums in
+// shared memory); an SM holds two blocks, the second one where more than half of them have a chunk
+// of the last round (3/8 after the first round, as measured: 109 ... 122 of 304); alone, a block
+// takes three quarters of a pair's time.  Projections and second projections of a step, cycles of
+// 96, us, FP64 form -> four or seven rows -> this: 300^2 200 -> 217 -> 193, 400^2 291 -> 343 -> 262,
+// 512^2 405 -> 347, 523^2 417 -> 486 -> 396, 560^2 465 -> 509 -> 431, 650^2 581 -> 636 -> 534.
+struct ProjShape { int rows, blocks; };
+static ProjShape proj_shape(long n) {
+    const long full = red_blocks();
+    ProjShape best{0, 0};
+    long least = 0;
+    for (int r = 3; r <= 7; r++) {
+        const long chunk = (long)r * kRedThreads, chunks = (n + chunk - 1) / chunk;
+        const long rounds = (chunks + full - 1) / full, last = chunks - (rounds - 1) * full;
+        const bool pair = last > (rounds == 1 ? full / 2 : 3 * full / 8);
+        const long cost = (r + 1) * (pair ? 4 * rounds : rounds == 1 ? 3 : 4 * rounds - 2);
+        if (best.rows == 0 || cost <= least) {
+            least = cost;
+            best = {r, (int)(chunks < full ? chunks : full)};
+        }
+    }
+    return best;
 }
 // Rows of the grid that share the groups of gv among nvt vectors: one, unless short vectors
 // leave SMs with fewer than 32 warps; then groups run side by side instead of one after
-// another.
+// another.  A full launch fills the SMs by its registers: a second row pays from eight groups on
+// (256^2, cycles of 128: 118 -> 112 us; of 16: 30.1 -> 31.5).
 static int red_rows(const RedShape& s, int nvt, int gv) {
     const int groups = (nvt + gv - 1) / gv;
+    if (s.threads == kRedThreads && groups < 8) return 1;
     const long warps = (long)s.blocks * (s.threads / 32), room = 16l * red_blocks();   // 32 warps per SM
     long y = room / warps;
     if (y > groups) y = groups;
@@ -1011,12 +1033,21 @@ die_status k_dots(const double2* V, long ldv, int nv, const double2* w, long n, 
     if (nv + 1 > kMaxBasis || nv < 0) return DIE_EINVAL;
     const RedShape sh = red_shape(n);
     const int nvt = nv + (with_norm ? 1 : 0);
-    if (VM && fix_rows(n))
-        DIE_PROF(PK_DOTS, st, launch_pdl(proj_rows(n) == 4 ? proj_fix_kernel<4> : proj_fix_kernel<7>, dim3(proj_blocks(n)), dim3(kRedThreads), 0, st, V, ldv, nv, w, n, with_norm, out, rs, skip, live ? 1 : 0));
-    else if (VM)
-        DIE_PROF(PK_DOTS, st, launch_pdl(proj3_kernel, dim3(sh.blocks, red_rows(sh, nvt, kGroup3)), dim3(sh.threads), 0, st, V, VM, ldv, nv, w, n, with_norm, out, rs, skip, live ? 1 : 0));
-    else
-        DIE_PROF(PK_DOTS, st, launch_pdl(proj_kernel<double2, kGroupFp64>, dim3(sh.blocks, red_rows(sh, nvt, kGroupFp64)), dim3(sh.threads), 0, st, V, ldv, nv, w, n, with_norm, out, rs, skip, live ? 1 : 0));
+    if (VM && fix_rows(n)) {
+        const ProjShape ps = proj_shape(n);
+        const auto kern = ps.rows == 3   ? proj_fix_kernel<3>
+                          : ps.rows == 4 ? proj_fix_kernel<4>
+                          : ps.rows == 5 ? proj_fix_kernel<5>
+                          : ps.rows == 6 ? proj_fix_kernel<6>
+                                         : proj_fix_kernel<7>;
+        DIE_PROF(PK_DOTS, st, launch_pdl(kern, dim3(ps.blocks), dim3(kRedThreads), 0, st, V, ldv, nv, w, n, with_norm, out, rs, skip, live ? 1 : 0));
+    } else if (VM) {
+        const int y = red_rows(sh, nvt, kGroup3);
+        DIE_PROF(PK_DOTS, st, launch_pdl(y > 1 ? proj3_kernel<true> : proj3_kernel<false>, dim3(sh.blocks, y), dim3(sh.threads), 0, st, V, VM, ldv, nv, w, n, with_norm, out, rs, skip, live ? 1 : 0));
+    } else {
+        const int y = red_rows(sh, nvt, kGroupFp64);
+        DIE_PROF(PK_DOTS, st, launch_pdl(y > 1 ? proj_kernel<double2, kGroupFp64, true> : proj_kernel<double2, kGroupFp64, false>, dim3(sh.blocks, y), dim3(sh.threads), 0, st, V, ldv, nv, w, n, with_norm, out, rs, skip, live ? 1 : 0));
+    }
     DIE_LAUNCH_CHECK();
     return DIE_OK;
 }
