@@ -121,8 +121,10 @@ __global__ void __launch_bounds__(512) k3_gx(OpDev<float> op, const float2* __re
 }
 
 // ----------------------------------------------------------------------- K3K1
+// At 256 and 512 (eight values per thread) 40 registers in place of 63, for half again the warps:
+// 256 x 1024, 8 products 74 -> 63 us; one product unchanged.
 template <typename IO, int LS>
-__global__ void __launch_bounds__(512) k3k1_gx(OpDev<float> op, float2* __restrict__ W, const IO* __restrict__ u,
+__global__ void __launch_bounds__(512, LS == 256 || LS == 512 ? 3 : 0) k3k1_gx(OpDev<float> op, float2* __restrict__ W, const IO* __restrict__ u,
                                                const float2* __restrict__ chir, float2* __restrict__ vbuf,
                                                const int* __restrict__ skip) {
     constexpr FxPlan p = gx_plan(LS);
@@ -222,13 +224,115 @@ __global__ void __launch_bounds__(P * (LS / gx_plan(LS).ept)) k2_gx(OpDev<float>
     }
 }
 
+// Two planes with both values of a column index in one thread (G threads per column), where the
+// first and the last radix agree: the last forward stage leaves a thread the values that the first
+// inverse stage wants, so the Green multiply stays in registers, and a twiddle or Green factor
+// is loaded once for both planes.  Large launches of k2_gx are bound by those loads and by its
+// shared-memory traffic: 256^2, per launch, one product 9.4 -> 8.2 us, 8 25.6 -> 20.9, 32
+// 83 -> 67 (the half-filled kernels of fft_fast.cuh at this length: 10.3, 23.5, 70).
+template <int EPT, int R>
+__device__ __forceinline__ void gx_stage2(float2 (&x)[EPT], float2 (&y)[EPT], int Ns, int t, int G,
+                                          const float2* __restrict__ tw) {
+#pragma unroll
+    for (int b = 0; b < EPT / R; b++) {
+        if (Ns > 1) {
+            const int k = mod_ns(t + b * G, Ns);
+#pragma unroll
+            for (int r = 1; r < R; r++) {
+                const float2 w = ld_tw(&tw[r * Ns + k - 1]);
+                x[b * R + r] = cmul(x[b * R + r], w);
+                y[b * R + r] = cmul(y[b * R + r], w);
+            }
+        }
+        gx_dft<R>(&x[b * R]);
+        gx_dft<R>(&y[b * R]);
+    }
+}
+template <int LS> __device__ __forceinline__ void gx_transform2(float2 (&x)[gx_plan(LS).ept], float2 (&y)[gx_plan(LS).ept],
+                                                                float2* bx, float2* by, const float2* tw, int t) {
+    constexpr FxPlan p = gx_plan(LS);
+    constexpr int EPT = p.ept, R0 = p.r0, R1 = p.r1, G = LS / EPT;
+    gx_stage2<EPT, R0>(x, y, 1, t, G, tw);
+    stage_store<float2, EPT, R0>(bx, x, LS, 1, t, G);
+    stage_store<float2, EPT, R0>(by, y, LS, 1, t, G);
+    __syncthreads();
+    int Ns = R0;
+#pragma unroll
+    for (int s = 1; s <= p.q; s++) {
+        stage_load<float2, EPT, R1>(bx, x, LS, t, G);
+        stage_load<float2, EPT, R1>(by, y, LS, t, G);
+        gx_stage2<EPT, R1>(x, y, Ns, t, G, tw);
+        __syncthreads();
+        if (s < p.q) {
+            stage_store<float2, EPT, R1>(bx, x, LS, Ns, t, G);
+            stage_store<float2, EPT, R1>(by, y, LS, Ns, t, G);
+            __syncthreads();
+        }
+        Ns *= R1;
+    }
+}
+template <int LS>
+__global__ void __launch_bounds__(LS / gx_plan(LS).ept) k2_gx_pair(OpDev<float> op, float2* __restrict__ W,
+                                                                   const int* __restrict__ skip) {
+    constexpr FxPlan p = gx_plan(LS);
+    constexpr int EPT = p.ept, G = LS / EPT, Q2 = LS / 2 + 1;
+    static_assert(p.r0 == p.r1, "registers of the last stage are those of the first");
+    pdl_wait();
+    if (block_flag(skip)) return;
+    W += blockIdx.y * op.ws;            // right-hand side of a batched product
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float2* buf0 = reinterpret_cast<float2*>(smem_raw);
+    float2* buf1 = buf0 + padded_len(LS);
+    const int t = threadIdx.x, k1 = blockIdx.x;
+    float2* col0 = W + (long)k1 * op.n2;
+    float2* col1 = W + ((long)op.M1 + k1) * op.n2;
+    const int h1 = op.M1 >> 1;
+    const int k1q = k1 <= h1 ? k1 : op.M1 - k1;
+    const bool neg1 = k1 > h1;
+    const long plane = (long)op.Q1 * Q2;
+    const float2* g = op.gq + (long)k1q * Q2;
+    float2 x[EPT], y[EPT];
+#pragma unroll
+    for (int e = 0; e < EPT; e++) {
+        const int j = fx_slot<EPT, p.r0>(e), idx = t + j * G;
+        const bool in = j < EPT / 2 && idx < op.n2;
+        x[e] = in ? col0[idx] : make_float2(0.f, 0.f);
+        y[e] = in ? col1[idx] : make_float2(0.f, 0.f);
+    }
+    gx_transform2<LS>(x, y, buf0, buf1, op.gx2, t);
+#pragma unroll
+    for (int e = 0; e < EPT; e++) {
+        const int k2 = t + fx_slot<EPT, p.r0>(e) * G;
+        const bool neg2 = k2 > LS / 2;
+        const int k2q = neg2 ? LS - k2 : k2;
+        float2 w = __ldg(&g[2 * plane + k2q]);
+        if (neg1 != neg2) w = make_float2(-w.x, -w.y);
+        const float2 a = cadd(cmul(__ldg(&g[k2q]), x[e]), cmul(w, y[e]));
+        const float2 b = cadd(cmul(w, x[e]), cmul(__ldg(&g[plane + k2q]), y[e]));
+        x[e] = make_float2(a.y, a.x);
+        y[e] = make_float2(b.y, b.x);
+    }
+    gx_transform2<LS>(x, y, buf0, buf1, op.gx2, t);
+#pragma unroll
+    for (int e = 0; e < EPT; e++) {
+        const int j = fx_slot<EPT, p.r1>(e), idx = t + j * G;
+        if (j < EPT / 2 && idx < op.n2) {
+            col0[idx] = make_float2(x[e].y, x[e].x);
+            col1[idx] = make_float2(y[e].y, y[e].x);
+        }
+    }
+}
+
 // --------------------------------------------------------------------- launch
 template <int LS> static Launch gx_rows_launch(const OpDev<float>& v, int nb) {
     constexpr int G = LS / gx_plan(LS).ept;
     // the operator's schedule where it has one (half_filled_rows); else fewer rows per block
     // while that leaves no SM with two blocks
     if (half_filled_rows(v)) {
-        const int h = v.tr ? v.tr : default_tile_rows_c64(LS);
+        int h = v.tr ? v.tr : default_tile_rows_c64(LS);
+        // batches at length 256: 64-byte segments once four blocks per SM are left (32 products at
+        // 128^2, K1 13.4 -> 12.1 us, K3K1 20.9 -> 18.6; 8 of them 8.2 -> 8.4, 10.2 -> 10.5)
+        if (LS == 256 && !v.tr && (long)v.n2 * v.planes * nb >= 8 * 4 * 152) h = 8;
         return Launch{dim3((v.n2 + h - 1) / h, v.planes, nb), dim3(h * G), (size_t)h * tile_stride(LS) * sizeof(float2)};
     }
     int TR = kGxTileRows;
@@ -257,6 +361,13 @@ void GxLaunch<LS>::k2(const OpDev<float>& v, float2* W, const int* skip, cudaStr
     static std::atomic<bool> a2{false}, a3{false};
     const Launch l{dim3(v.M1, nb), dim3(v.planes * (LS / gx_plan(LS).ept)),
                    (size_t)v.planes * padded_len(LS) * sizeof(float2)};
+    if constexpr (LS == 512) {     // equal radices; other such lengths are short or fast_length
+        static std::atomic<bool> ap{false};
+        if (v.planes == 2) {
+            launch_kernel(k2_gx_pair<LS>, ap, Launch{l.grid, dim3(LS / gx_plan(LS).ept), l.smem}, st, v, W, skip);
+            return;
+        }
+    }
     if (v.planes == 3) launch_kernel(k2_gx<3, LS>, a3, l, st, v, W, skip);
     else launch_kernel(k2_gx<2, LS>, a2, l, st, v, W, skip);
 }
