@@ -329,7 +329,6 @@ static die_status create_impl(const dieop_desc* desc, const void* eps_r, int eps
     DIE_TRY(dmalloc(&op->ws.v, op->ws.v_bytes));
     DIE_TRY(dmalloc(&op->dflag, sizeof(int)));
     DIE_CUDA_TRY(cudaMemsetAsync(op->dflag, 0, sizeof(int), st));
-    DIE_TRY(set_kernel_attributes(op));
 
     std::vector<double2> t1d, t2d;
     std::vector<float2> t1f, t2f;

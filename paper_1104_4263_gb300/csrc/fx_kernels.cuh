@@ -180,44 +180,39 @@ template <int EPT, int R0, int R1, int LS>
 __device__ __forceinline__ void fx_transform(fxc (&x)[EPT], fxc* buf, int q, const fxw* tw, int t, int G, int L,
                                              FxScale& sc) {
     fx_first<EPT, R0>(x);
-    constexpr bool kSingle = LS == R0;
-    if constexpr (!kSingle) {
-        stage_store<fxc, EPT, R0>(buf, x, L, 1, t, G);
-        __syncthreads();
-        int Ns = R0, room = 0;
-        const bool rise = q > 1 && !sc.bad;
-        if (rise) room = fx_room(R0, R1, q, sc.half, sc.lm, sc.ls, 0);
-        auto stage = [&](int s) {
-            stage_load<fxc, EPT, R1>(buf, x, L, t, G);
-            if (rise && s > 1) {
-                const int to = fx_room(R0, R1, q, sc.half, sc.lm, sc.ls, s - 1);
-                const int up = max(0, min(to - room, 31));
-                room = to;
-                if (up) {
+    stage_store<fxc, EPT, R0>(buf, x, L, 1, t, G);
+    __syncthreads();
+    int Ns = R0, room = 0;
+    const bool rise = q > 1 && !sc.bad;
+    if (rise) room = fx_room(R0, R1, q, sc.half, sc.lm, sc.ls, 0);
+    auto stage = [&](int s) {
+        stage_load<fxc, EPT, R1>(buf, x, L, t, G);
+        if (rise && s > 1) {
+            const int to = fx_room(R0, R1, q, sc.half, sc.lm, sc.ls, s - 1);
+            const int up = max(0, min(to - room, 31));
+            room = to;
+            if (up) {
 #pragma unroll
-                    for (int e = 0; e < EPT; e++) x[e] = fxc{fx_shl(x[e].x, up), fx_shl(x[e].y, up)};
-                    sc.e += up;
-                }
+                for (int e = 0; e < EPT; e++) x[e] = fxc{fx_shl(x[e].x, up), fx_shl(x[e].y, up)};
+                sc.e += up;
             }
-            fx_stage<EPT, R1>(x, Ns, t, G, tw);
-            __syncthreads();
-            if (s == q) return;
-            stage_store<fxc, EPT, R1>(buf, x, L, Ns, t, G);
-            __syncthreads();
-            Ns *= R1;
-        };
-        if constexpr (LS != 0 && R1 == 4) {       // short stages, Ns = 3 * 2^b: divisions by constants
-#pragma unroll
-            for (int s = 1; s <= fx_plan(LS ? LS : 16).q; s++) stage(s);
-        } else {
-#pragma unroll 1
-            for (int s = 1; s <= q; s++) stage(s);
         }
-        sc.e -= 2 * q;
+        fx_stage<EPT, R1>(x, Ns, t, G, tw);
+        __syncthreads();
+        if (s == q) return;
+        stage_store<fxc, EPT, R1>(buf, x, L, Ns, t, G);
+        __syncthreads();
+        Ns *= R1;
+    };
+    if constexpr (LS != 0 && R1 == 4) {       // short stages, Ns = 3 * 2^b: divisions by constants
+#pragma unroll
+        for (int s = 1; s <= fx_plan(LS ? LS : 16).q; s++) stage(s);
+    } else {
+#pragma unroll 1
+        for (int s = 1; s <= q; s++) stage(s);
     }
+    sc.e -= 2 * q;
 }
-// Last radix of a plan.
-template <int R0, int R1, int LS> constexpr int fx_last() { return LS == R0 ? R0 : R1; }
 
 template <int EPT> __device__ __forceinline__ void fx_swap(fxc (&x)[EPT]) {
 #pragma unroll
@@ -229,7 +224,7 @@ template <int EPT> __device__ __forceinline__ void fx_swap(fxc (&x)[EPT]) {
 template <int EPT, int R0, int R1, int LS>
 __device__ __forceinline__ void fx_row_forward(double2 (&z)[EPT], fxc* buf, const FxDev& op, int t, int G, int L,
                                                FxNorm* red) {
-    constexpr int RL = fx_last<R0, R1, LS>();
+    constexpr int RL = R1;
     auto low = [](int e) { return fx_slot<EPT, R0>(e) < EPT / 2; };
     const int q = LS ? fx_plan(LS ? LS : 16).q : op.q1;
     FxScale s = fx_scale(fx_group_norm(fx_norm<EPT>(z, low), G, red), R0, R1, q, true);
@@ -246,7 +241,7 @@ __device__ __forceinline__ void fx_row_forward(double2 (&z)[EPT], fxc* buf, cons
 template <int EPT, int R0, int R1, int LS>
 __device__ __forceinline__ void fx_row_inverse(fxc* buf, double2 (&y)[EPT], const FxDev& op, int t, int G, int L,
                                                FxNorm* red) {
-    constexpr int RL = fx_last<R0, R1, LS>();
+    constexpr int RL = R1;
     auto all = [](int) { return true; };
     const int q = LS ? fx_plan(LS ? LS : 16).q : op.q1;
     double2 z[EPT];
@@ -320,7 +315,7 @@ __global__ void __launch_bounds__(512) k1_fx(FxDev op, const double2* u, const d
 template <int EPT, int R0, int R1, int LS>
 __global__ void __launch_bounds__(512) k3_fx(FxDev op, const double2* __restrict__ W, const double2* __restrict__ u,
                                              double2* __restrict__ y, const int* __restrict__ skip) {
-    constexpr int RL = fx_last<R0, R1, LS>();
+    constexpr int RL = R1;
     __shared__ FxNorm red[16];
     pdl_wait();
     if (block_flag(skip)) return;
@@ -348,7 +343,7 @@ template <int EPT, int R0, int R1, int LS>
 __global__ void __launch_bounds__(512) k3k1_fx(FxDev op, double2* __restrict__ W, const double2* __restrict__ u,
                                                const double2* __restrict__ chir, double2* __restrict__ vbuf,
                                                const int* __restrict__ skip) {
-    constexpr int RL = fx_last<R0, R1, LS>();
+    constexpr int RL = R1;
     __shared__ FxNorm red[16], red2[16];
     pdl_wait();
     if (block_flag(skip)) return;
@@ -414,7 +409,7 @@ constexpr int fx_k2_blocks(int threads, int ept) {
 
 template <int P, int EPT, int R0, int R1, int LS, int MAXT>
 __global__ void __launch_bounds__(MAXT, fx_k2_blocks(MAXT, EPT)) k2_fx(FxDev op, double2* __restrict__ W, const int* __restrict__ skip) {
-    constexpr int RL = fx_last<R0, R1, LS>();
+    constexpr int RL = R1;
     __shared__ FxNorm red[32], redp[2][3];
     pdl_wait();
     if (block_flag(skip)) return;

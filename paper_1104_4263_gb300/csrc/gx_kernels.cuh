@@ -361,15 +361,13 @@ void GxLaunch<LS>::k2(const OpDev<float>& v, float2* W, const int* skip, cudaStr
     static std::atomic<bool> a2{false}, a3{false};
     const Launch l{dim3(v.M1, nb), dim3(v.planes * (LS / gx_plan(LS).ept)),
                    (size_t)v.planes * padded_len(LS) * sizeof(float2)};
-    if constexpr (LS == 512) {     // equal radices; other such lengths are short or fast_length
-        static std::atomic<bool> ap{false};
-        if (v.planes == 2) {
-            launch_kernel(k2_gx_pair<LS>, ap, Launch{l.grid, dim3(LS / gx_plan(LS).ept), l.smem}, st, v, W, skip);
-            return;
-        }
+    if (v.planes == 3) {
+        launch_kernel(k2_gx<3, LS>, a3, l, st, v, W, skip);
+    } else if constexpr (LS == 512) {     // equal radices; other such lengths are short or fast_length
+        launch_kernel(k2_gx_pair<LS>, a2, Launch{l.grid, dim3(LS / gx_plan(LS).ept), l.smem}, st, v, W, skip);
+    } else {
+        launch_kernel(k2_gx<2, LS>, a2, l, st, v, W, skip);
     }
-    if (v.planes == 3) launch_kernel(k2_gx<3, LS>, a3, l, st, v, W, skip);
-    else launch_kernel(k2_gx<2, LS>, a2, l, st, v, W, skip);
 }
 
 // Instantiates the launchers of one length.

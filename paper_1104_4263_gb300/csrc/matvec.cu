@@ -34,9 +34,6 @@ OpDev<float> view_f(const dieop_s* op) {
     return v;
 }
 
-// Shared-memory limits are raised lazily by each launcher on first use.
-die_status set_kernel_attributes(const dieop_s*) { return DIE_OK; }
-
 // Calls f with the launchers of a transform length.
 template <typename F> static void fx_for_length(int L, F&& f) {
     switch (L) {

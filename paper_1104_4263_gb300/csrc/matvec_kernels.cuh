@@ -35,8 +35,8 @@
 namespace die {
 
 // Rows per block of the row passes: enough for 32-byte segments in the transposed
-// accesses (4 complex64), at most 512 threads per block.
-template <typename C> constexpr int tile_rows() { return sizeof(C) == 8 ? 4 : 2; }
+// accesses, at most 512 threads per block.
+constexpr int kTileRows = 4;
 // The column pass stages its Green spectra where that leaves room for two blocks per SM
 // (not at length 4096: 119 KB with them, 70 KB without; two blocks of 128 registers there:
 // product at 2048^2 770 -> 704 us).
@@ -61,12 +61,12 @@ __device__ __forceinline__ void load_tile(C* tile, const C* __restrict__ W, int 
 }
 
 // ------------------------------------------------------------------ fast path
-// Grids with n = L / 2 exactly and L = 2^a in [256, 4096] (the padding is then exactly
-// half of every transform): the same passes with the compile-time stages of
-// fft_fast.cuh.  The zero inputs (index >= n) of the forward transforms and the
-// discarded outputs (index >= n) of the inverse ones are known at compile time.
+// Transforms of length L = 1024, 2048 and 4096 (the deflated first row pass: 2^a from 256 on) with
+// the compile-time stages of fft_fast.cuh.  The zero inputs (index >= L / 2) of the forward
+// transforms and the discarded outputs of the inverse ones are known at compile time; a grid
+// that fills less than half of a transform (RAG) checks the others' indices.
 template <typename C, int L> constexpr int fast_tr() {
-    return tile_rows<C>() * (L / 16) <= kRowsMaxThreads ? tile_rows<C>() : kRowsMaxThreads / (L / 16);
+    return kTileRows * (L / 16) <= kRowsMaxThreads ? kTileRows : kRowsMaxThreads / (L / 16);
 }
 template <int L> constexpr int tile_stride_c() { return L + (L >> 4) + 2; }
 
@@ -459,8 +459,8 @@ inline void launch_kernel(K kernel, std::atomic<bool>& attr_set, const Launch& l
 
 // Transforms on the stages of fft_fast.cuh: two planes, L = 1024, 2048 or 4096 (16 values per
 // thread, both components of a column in one thread).  Shorter ones, 3 * 2^a and three planes
-// take the any-grid kernels (gx_kernels.cuh), which are faster there: 128^2 22.3 -> 19 us,
-// 256^2 27 -> 24; at L = 1024 they take 62 us where these take 46.
+// take the any-grid kernels (gx_kernels.cuh), which are faster there: 128^2 24.3 -> 20 us,
+// 256^2 29 -> 23; at L = 1024 they take 62 us where these take 46.
 inline bool fast_length(int L) { return L == 1024 || L == 2048 || L == 4096; }
 template <typename T> inline bool fast_rows(const OpDev<T>& v) { return v.planes == 2 && fast_length(v.M1); }
 template <typename T> inline bool fast_cols(const OpDev<T>& v) { return v.planes == 2 && fast_length(v.M2); }
@@ -489,8 +489,8 @@ template <typename C, int L, int TR> inline Launch rows_launch_fast(int n2) {
         default: DIE_FAST_SWITCH(M, CASE); break; \
     }
 
-// Tile height of the fast row passes: the rows of one block (TR).  0 selects fast_tr,
-// the default of the element type and length; an operator's schedule (dieop_autotune,
+// Tile height of the fast row passes: the rows of one block (TR).  0 selects fast_tr, the
+// default of the length; an operator's schedule (dieop_autotune,
 // dieop_set_tile_rows) may pick another valid height for its complex64 passes.  Every row
 // is transformed by the same threads and stages whatever TR is, so the products are
 // bit-identical for all heights.
@@ -512,18 +512,15 @@ template <int TR>
 void rows_defl_fast(const OpDev<float>& v, const DeflIn& d, const float2* chi, float2* z, float2* W, const int* skip,
                     cudaStream_t st);
 
-// Calls F<TR> with the tile height of the view (complex64: the operator's schedule).
+// Calls F<TR> with the tile height of the view (the operator's schedule).
 template <typename T, typename F>
 inline void with_tile_rows(const OpDev<T>& v, F&& f) {
-    if constexpr (sizeof(C_t<T>) == 8) {
-        switch (tile_rows_code(v.tr, v.M1)) {
-            case 1: f(std::integral_constant<int, 1>{}); return;
-            case 2: f(std::integral_constant<int, 2>{}); return;
-            case 8: f(std::integral_constant<int, 8>{}); return;
-            default: break;
-        }
+    switch (tile_rows_code(v.tr, v.M1)) {
+        case 1: f(std::integral_constant<int, 1>{}); return;
+        case 2: f(std::integral_constant<int, 2>{}); return;
+        case 8: f(std::integral_constant<int, 8>{}); return;
+        default: f(std::integral_constant<int, 0>{});
     }
-    f(std::integral_constant<int, 0>{});
 }
 
 // nb > 1: a batched product over nb right-hand sides (grid z: row passes, grid y: columns).

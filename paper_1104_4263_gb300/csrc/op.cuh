@@ -149,6 +149,5 @@ bool defl_product_ok(const dieop_s* op);
 die_status apply_defl_xy(dieop_s* op, const DeflIn& d, float2* z, double2* y, bool reg, const int* skip,
                          cudaStream_t st, const Workspace* ws = nullptr);
 
-die_status set_kernel_attributes(const dieop_s* op);
 
 }  // namespace die
