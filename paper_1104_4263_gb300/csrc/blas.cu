@@ -594,10 +594,12 @@ __device__ __forceinline__ void fix_update(const double2* __restrict__ V, long l
 // out = base + sum_i V_i c_i.  Coefficients: c = sign * coef, or c = M s when M != NULL.
 // The sum for a row starts from base and runs through the basis in order in one pair of
 // accumulators (the FP64 pipe, not the FMA latency, bounds the loop).
-// FIX: the fixed-point form, at two blocks per SM (no bound otherwise: with one of 1 the compiler
-// takes 82 registers for 48, and the deflation update of 9 vectors at 512^2 45 us for 41).
+// FIX: the fixed-point form, at two blocks per SM.  The FP64 form with a norm (Gram-Schmidt) has a
+// bound of one, which makes the compiler take 83 registers for 54 (cycles of 150 at 133^2: 75 us for
+// 84 a step), the one without has none (82 for 48 registers: the deflation update of 9 vectors at
+// 512^2 45 us for 41).
 template <typename VT, bool NORM, bool FIX>
-__global__ void __launch_bounds__(kRedThreads, FIX ? 2 : 0) basis_axpy_kernel(const VT* __restrict__ V, long ldv, int k,
+__global__ void __launch_bounds__(kRedThreads, FIX ? 2 : NORM ? 1 : 0) basis_axpy_kernel(const VT* __restrict__ V, long ldv, int k,
                                                                  const double2* __restrict__ coef, double sign,
                                                                  const double2* __restrict__ M,
                                                                  const double2* __restrict__ s, const double2* base,
@@ -699,8 +701,10 @@ __global__ void __launch_bounds__(kRedThreads, FIX ? 2 : 0) basis_axpy_kernel(co
 // pass).  Reduction vector 0 is ||w||^2, vectors 1 .. r the projections.  The last
 // block writes ||w||^2 to nrm2 and, when no second pass follows, 1 / ||w|| to dec.inv
 // and cf = M32 (V32^* w / ||w||) to dp.cf.
+// Up to 16 deflation vectors the FP64 form has the bound of one that basis_axpy_kernel has; beyond,
+// it would take more than 128 registers (20 vectors at 256^2: 41 us for 33).
 template <int NGD, bool FIX>
-__global__ void __launch_bounds__(kRedThreads, FIX ? 2 : 0) cgs_update_defl_kernel(const double2* __restrict__ V, long ldv, int k,
+__global__ void __launch_bounds__(kRedThreads, FIX ? 2 : NGD <= 2 ? 1 : 0) cgs_update_defl_kernel(const double2* __restrict__ V, long ldv, int k,
                                                                       const double2* __restrict__ coef,
                                                                       const double2* base, double2* out, long n,
                                                                       double2* nrm2, Dgks dec, int has_dec,
