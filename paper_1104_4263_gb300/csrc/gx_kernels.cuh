@@ -271,6 +271,15 @@ template <int LS> __device__ __forceinline__ void gx_transform2(float2 (&x)[gx_p
         Ns *= R1;
     }
 }
+// a u + b v, each product rounded before the sum (no multiply-add across it): the results are those
+// of k2_gx to the bit.
+__device__ __forceinline__ float2 gx_green(float2 a, float2 u, float2 b, float2 v) {
+    auto mul = [](float2 p, float2 q) {
+        return make_float2(__fmaf_rn(p.x, q.x, -__fmul_rn(p.y, q.y)), __fmaf_rn(p.x, q.y, __fmul_rn(p.y, q.x)));
+    };
+    const float2 x = mul(a, u), y = mul(b, v);
+    return make_float2(__fadd_rn(x.x, y.x), __fadd_rn(x.y, y.y));
+}
 template <int LS>
 __global__ void __launch_bounds__(LS / gx_plan(LS).ept) k2_gx_pair(OpDev<float> op, float2* __restrict__ W,
                                                                    const int* __restrict__ skip) {
@@ -307,8 +316,8 @@ __global__ void __launch_bounds__(LS / gx_plan(LS).ept) k2_gx_pair(OpDev<float> 
         const int k2q = neg2 ? LS - k2 : k2;
         float2 w = __ldg(&g[2 * plane + k2q]);
         if (neg1 != neg2) w = make_float2(-w.x, -w.y);
-        const float2 a = cadd(cmul(__ldg(&g[k2q]), x[e]), cmul(w, y[e]));
-        const float2 b = cadd(cmul(w, x[e]), cmul(__ldg(&g[plane + k2q]), y[e]));
+        const float2 a = gx_green(__ldg(&g[k2q]), x[e], w, y[e]);
+        const float2 b = gx_green(w, x[e], __ldg(&g[plane + k2q]), y[e]);
         x[e] = make_float2(a.y, a.x);
         y[e] = make_float2(b.y, b.x);
     }
