@@ -594,12 +594,12 @@ __device__ __forceinline__ void fix_update(const double2* __restrict__ V, long l
 // out = base + sum_i V_i c_i.  Coefficients: c = sign * coef, or c = M s when M != NULL.
 // The sum for a row starts from base and runs through the basis in order in one pair of
 // accumulators (the FP64 pipe, not the FMA latency, bounds the loop).
-// FIX: the fixed-point form, at two blocks per SM.  The FP64 form with a norm (Gram-Schmidt) has a
-// bound of one, which makes the compiler take 83 registers for 54 (cycles of 150 at 133^2: 75 us for
-// 84 a step), the one without has none (82 for 48 registers: the deflation update of 9 vectors at
-// 512^2 45 us for 41).
-template <typename VT, bool NORM, bool FIX>
-__global__ void __launch_bounds__(kRedThreads, FIX ? 2 : NORM ? 1 : 0) basis_axpy_kernel(const VT* __restrict__ V, long ldv, int k,
+// FIX: the fixed-point form.  MINB: blocks per SM that the registers are bounded for: two in fixed
+// point; one in the FP64 sweeps over a Krylov basis, which makes the compiler take 83 registers for
+// 54 (cycles of 150 at 133^2: 75 us for 84 a step); no bound (0) in the deflation update (82 for
+// 48 registers: 9 vectors at 512^2 45 us for 41).
+template <typename VT, bool NORM, bool FIX, int MINB = FIX ? 2 : 1>
+__global__ void __launch_bounds__(kRedThreads, MINB) basis_axpy_kernel(const VT* __restrict__ V, long ldv, int k,
                                                                  const double2* __restrict__ coef, double sign,
                                                                  const double2* __restrict__ M,
                                                                  const double2* __restrict__ s, const double2* base,
@@ -1076,7 +1076,9 @@ die_status k_basis_axpy(const double2* V, long ldv, int k, const double2* coef, 
                      V, ldv, k, coef, sign, (const double2*)nullptr, (const double2*)nullptr, base, out, n, nrm2, d, has_dec, rs, skip, live ? 1 : 0, VM));
     } else {
         const int t = axpy_threads(n);
-        const auto kern = VM && fix_rows(n) ? basis_axpy_kernel<double2, false, true> : basis_axpy_kernel<double2, false, false>;
+        const auto kern = !VM           ? basis_axpy_kernel<double2, false, false, 0>
+                          : fix_rows(n) ? basis_axpy_kernel<double2, false, true>
+                                        : basis_axpy_kernel<double2, false, false>;
         DIE_PROF(PK_LINCOMB, st, launch_pdl(kern, dim3(grid_for(n, t)), dim3(t), 0, st,
                      V, ldv, k, coef, sign, (const double2*)nullptr, (const double2*)nullptr, base, out, n, (double2*)nullptr, d, 0, rs, skip, 0, VM));
     }
@@ -1087,7 +1089,7 @@ die_status k_defl_update(const double2* V, long ldv, int r, const double2* M, co
                          double2* z, long n, const int* skip, cudaStream_t st) {
     if (r > kMaxBasis || r < 1) return DIE_EINVAL;
     const int t = axpy_threads(n);
-    DIE_PROF(PK_DEFL_UPDATE, st, launch_pdl(basis_axpy_kernel<double2, false, false>, dim3(grid_for(n, t)), dim3(t), 0, st,
+    DIE_PROF(PK_DEFL_UPDATE, st, launch_pdl(basis_axpy_kernel<double2, false, false, 0>, dim3(grid_for(n, t)), dim3(t), 0, st,
                  V, ldv, r, (const double2*)nullptr, 1.0, M, s, x, z, n, (double2*)nullptr, Dgks{}, 0, RedScratch{}, skip, 0, (const double*)nullptr));
     DIE_LAUNCH_CHECK();
     return DIE_OK;
