@@ -52,18 +52,29 @@ UNIT = "regularized matvecs/s"
 WORKLOAD = ("core-shell 512x512 (eps -2+0.1i core R1.5, 20+0.5i shell R2.5, side 8): A_R A P^-1, GMRES(30), r=20, "
             "FP32 products + FP64 Krylov, 1500 Arnoldi steps per step")
 L2_NOTE = "working set > L2 (Krylov basis 31 x 8.4 MB, deflation basis 20 x 4.2 MB)"
-# ncu DRAM bytes (read + write) of one launch of the FP64 projection kernel on this
-# workload: 13 basis vectors (16 B a value) and the norm of w, over 2N = 524288, from one
-# capture of the committed profile driver (bench.py --profile-driver).  Its traffic grows with the vectors
-# read, so it is scaled to the bench's average launch by the algorithmic bytes.
 # DRAM bytes of the five passes of one complex64 regularised product at 512^2 (reads; no
 # DRAM writes were counted during the passes: the row spectra stay in L2)
 NCU_PRODUCT = {"dram_bytes": (6.315520 + 14.774016 + 14.725632 + 14.769408 + 12.608512) * 1e6, "n": 524288,
                "source": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum -k regex:\"k1_fast|k2_fast2|"
                          "k3k1_fast|k3_fast\" -c 5 on bench.py --profile-driver (its first complex64 product)"}
-NCU_DOTS = {"dram_bytes": 118.963456e6 + 3.052032e6, "nv": 13, "n": 524288,
-            "source": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum -k regex:proj_fix on "
-                      "bench.py --profile-driver (the 13-vector launch; groups of seven vectors)"}
+# ncu DRAM bytes (read + write) of one launch of the Gram-Schmidt sweeps on this workload, over
+# 2N = 524288, from captures of the committed profile driver (bench.py --profile-driver): the
+# projections on 13 basis vectors (16 B a value) and the norm of w; the update over 16 with the
+# 20 complex64 deflation projections.  Their traffic grows with the vectors read, so it is scaled
+# to the bench's average launch by the algorithmic bytes ("alg": bytes per element of the launch).
+NCU_SWEEPS = {
+    "dots": {"dram_bytes": 118.963456e6 + 3.052032e6, "alg": 13 * 16 + 16, "n": 524288,
+             "source": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum -k regex:proj_fix on "
+                       "bench.py --profile-driver (the 13-vector launch; groups of eight vectors, seven rows "
+                       "per thread)"},
+    "cgs_update_norm": {"dram_bytes": 226.610944e6 + 7.426048e6, "alg": 16 * 16 + 32 + 20 * 8, "n": 524288,
+                        "source": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum -k regex:cgs_update_defl "
+                                  "on bench.py --profile-driver (the 16-vector launch)"},
+}
+# Vectors of more than two rows per thread of a full launch (two blocks of 256 threads on each of
+# 152 SMs): the Gram-Schmidt sweeps run in fixed point.  Integer instructions bound them, for
+# which there is no peak to divide by, so their roofline is the one left, HBM.
+FIXED_POINT_FROM = 2 * 2 * 152 * 256
 
 
 def fp64_peak(die):
@@ -273,6 +284,13 @@ def work_model(cls, p, op, r, steps_per_cycle, cycles, products, fp64_products):
         # deflation projections (r vectors + x)
         per_cycle = sum((j + 1) * 16 + 16 for j in range(m)) + 16 + 16 * r + 16
         return "hbm", cycles * per_cycle * n + 16 * n
+    if cls == "dots" and n > FIXED_POINT_FROM:
+        return work_model("dots_bytes", p, op, r, steps_per_cycle, cycles, products, fp64_products)
+    if cls == "cgs_update_norm" and n > FIXED_POINT_FROM:
+        # step j: j+1 basis vectors, w read and written, and (folded in up to rank 32) the
+        # complex64 deflation basis
+        per_cycle = sum((j + 1) * 16 + 32 + (8 * r if r <= 32 else 0) for j in range(m))
+        return "hbm", cycles * per_cycle * n
     if cls == "dots":
         # step j of a cycle: j+1 projections + the norm of w; per cycle one norm of the
         # residual, one FP64 deflation projection set (r) for the update of x
@@ -494,20 +512,17 @@ def main():
                                "unit": "GB/s", "frac": (per_launch / avg_s / 1e9) / hbm_peak, "traffic": None,
                                "kernel": best, "algorithmic_bytes_per_launch": per_launch,
                                "peak_source": "MEASURED_PEAKS.json hbm_gbs" if peaks else "fallback"}
+            cap = NCU_SWEEPS.get(best)
+            if cap and 2 * p.N == cap["n"] > FIXED_POINT_FROM:
+                out["roofline"]["traffic"] = cap["dram_bytes"] * per_launch / (cap["alg"] * cap["n"])
+                out["roofline"]["traffic_source"] = (cap["source"] + ", scaled to the average launch by the "
+                                                     "algorithmic bytes")
         else:
             out["roofline"] = {"bound": "alu", "achieved": per_launch / avg_s / 1e12, "peak": FP64_PEAK_TFLOPS,
                                "unit": "TFLOP/s", "frac": (per_launch / avg_s / 1e12) / FP64_PEAK_TFLOPS,
                                "traffic": None, "kernel": best, "algorithmic_flops_per_launch": per_launch,
                                "peak_source": (f"FP64 FMA probe of this run (die_fp64_peak, {fp64['sms']} SMs; "
                                                f"nominal {fp64['nominal_tflops']:.3f} TFLOP/s)")}
-            if best == "dots" and NCU_DOTS and 2 * p.N == NCU_DOTS["n"]:
-                _, tot_bytes = work_model("dots_bytes", p, op, D.r, RESTART, cycles, prof_products, fp64_products)
-                alg_bytes = tot_bytes / k["launches"]
-                captured_alg = (NCU_DOTS["nv"] * 16 + 16) * NCU_DOTS["n"]
-                out["roofline"]["traffic"] = NCU_DOTS["dram_bytes"] * alg_bytes / captured_alg
-                out["roofline"]["algorithmic_bytes_per_launch"] = alg_bytes
-                out["roofline"]["traffic_source"] = (NCU_DOTS["source"] + ", scaled to the average launch by the "
-                                                     "algorithmic bytes")
 
     _extra(out, "matvec", lambda: matvec_rates(op, p, die, torch))
     if isinstance(out.get("matvec"), dict) and "c64" in out["matvec"]:

@@ -290,13 +290,17 @@ __global__ void __launch_bounds__(kRedThreads, 2) proj3_kernel(const double2* __
 // ----------------------------------------------------- fixed-point Gram-Schmidt sweeps
 // The update w - V h is a sum of products of FP64 numbers; GB300's FP64 pipe does 2 FMAs per
 // clock and SM, its integer pipes 24 32 x 32 -> 64-bit multiply-adds.  So a row's eight basis
-// values (of a common exponent) and their coefficients are brought to 58-bit integers, the
-// products accumulated exactly but for the bits below 2^32 of their 118, and only the sums of
-// eight terms go through the FP64 pipe (4 operations instead of 24).  A term's error is 2^-58
-// of the largest term of its sum, below the 2^-53 of every term in FP64.  Complex products take
-// Gauss's three multiplications.  At 512^2 (cylinder, r = 8, 15 vectors on average) the update
-// takes 62 us where the FP64 form takes 92, bound by the conversions; the projections
-// (proj_fix_kernel), where a thread's rows share the exponent, 64 us for 75.
+// values (of a common exponent) and the coefficients (one exponent for all of an update) are
+// brought to 58-bit integers, the products accumulated exactly but for the bits below 2^32 of
+// their 118, and only the sums of eight terms go through the FP64 pipe (4 operations instead of
+// 24).  In the projections the rows of a thread share the exponents, of w's values and of each
+// vector's.  An operand is cut to 2^-58 of its group's bound: a term's error is some 2^-57 of the
+// two bounds' product.  That is normwise below the 2^-53 per term of the FP64 form (orthogonality
+// and residuals as before), but not against a small term beside a large value of its group: a
+// value 2^5 below the largest keeps 53 bits, one 2^58 below none.  Complex products take Gauss's
+// three multiplications.  At 512^2 (cylinder, r = 8, 15 vectors on average) the update takes
+// 62 us where the FP64 form takes 92, bound by the conversions; the projections
+// (proj_fix_kernel) 64 us for 75.
 constexpr int kGsBits = 58;                  // |operand| < 2^58, sums and differences < 2^59
 // Least common exponent field of a group of operands: from 2^-958 of its bound down, a value
 // counts in units of 2^-1016, so that zeros (field 0, no leading bit) shift out whole.

@@ -6,7 +6,7 @@
 // thread (the FP64 forms were bound by the FP64 pipe).  CUDA-event times per launch, FP64
 // form -> this one: 512^2 K1 82.5 -> 29.6 us, K2 290.6 -> 66.2, K3K1 155.5 -> 45.0, K3
 // 79.8 -> 26.5 (the regularised product 878 -> 207 us back to back); 61^2 128 -> 44 us; the
-// three-plane product at 384^2 476 -> 132 us.  Lengths 3 * 2^a have compile-time plans from
+// three-plane product at 384^2 476 -> 123 us.  Lengths 3 * 2^a have compile-time plans from
 // 48 to 1536 (runtime -> compile time: 96^2 83 -> 61 us, 700^2 700 -> 563).  A product's own rounding (spread of
 // y(c x) / c over random factors c) is 3.2e-16 ... 3.9e-16 of it at 61^2 ... 2048 x 1500 on
 // noise and wave fields, against 3.5e-16 ... 3.8e-16 of the FP64 form, and 3.3e-16 ...

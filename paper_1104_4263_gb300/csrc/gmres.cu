@@ -431,7 +431,8 @@ static die_status solve_ctx(dieop_s* op, defl_s* defl, const gmres_opts* o, cons
     const bool fold_product = fold && defl_product_ok(op);   // deflation inside the first row pass
     // Update passes in the three-multiplication form: every kernel that normalises a basis
     // vector also stores its Re - Im in c->Vm (all paths but the separate complex64
-    // projection pass of r > kDeflFoldMax).
+    // projection pass of r > kDeflFoldMax).  The sweeps over long vectors take its presence as
+    // the choice of their fixed-point form and do not read it.
     double* Vm = (defl32 && !fold) ? nullptr : c->Vm;
     DeflProj dp;
     if (fold) {
