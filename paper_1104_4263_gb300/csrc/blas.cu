@@ -992,7 +992,7 @@ static bool fix_rows(long n) { return n > 2l * red_blocks() * kRedThreads; }
 // Rows per thread and chunk, and blocks, of the fixed-point projections: the rows that leave the
 // busiest SM the least to do.  A chunk costs its rows and about one more (its exponent, the sums in
 // shared memory); an SM holds two blocks, the second one where more than half of them have a chunk
-// of the last round (3/8 after the first round, as measured: 109 ... 122 of 304); alone, a block
+// in the blocks' last turn (3/8 after the first turn, as measured: 109 ... 122 of 304); alone, a block
 // takes three quarters of a pair's time.  Projections and second projections of a step, cycles of
 // 96, us, FP64 form -> four or seven rows -> this: 300^2 200 -> 217 -> 193, 400^2 291 -> 343 -> 262,
 // 512^2 405 -> 347, 523^2 417 -> 486 -> 396, 560^2 465 -> 509 -> 431, 650^2 581 -> 636 -> 534.
@@ -1003,9 +1003,9 @@ static ProjShape proj_shape(long n) {
     long least = 0;
     for (int r = 3; r <= 7; r++) {
         const long chunk = (long)r * kRedThreads, chunks = (n + chunk - 1) / chunk;
-        const long rounds = (chunks + full - 1) / full, last = chunks - (rounds - 1) * full;
-        const bool pair = last > (rounds == 1 ? full / 2 : 3 * full / 8);
-        const long cost = (r + 1) * (pair ? 4 * rounds : rounds == 1 ? 3 : 4 * rounds - 2);
+        const long turns = (chunks + full - 1) / full, last = chunks - (turns - 1) * full;
+        const bool pair = last > (turns == 1 ? full / 2 : 3 * full / 8);
+        const long cost = (r + 1) * (pair ? 4 * turns : turns == 1 ? 3 : 4 * turns - 2);
         if (best.rows == 0 || cost <= least) {
             least = cost;
             best = {r, (int)(chunks < full ? chunks : full)};
